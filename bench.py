@@ -58,7 +58,12 @@ FP32_LANES_PER_SM = 128
 FP64_TFLOPS_NOMINAL = 1.25
 TF32_PER_BF16 = 1.1 / 2.25
 TF32_SPLIT_TERMS = 3      # a_hi b_hi + a_hi b_lo + a_lo b_hi per FP32-accurate product
-DF_INSTR_PER_CMAC = 48     # FP32 instructions of one double-float complex multiply-add (near field)
+# near field on the tensor cores: FP16 multiply-adds of one complex multiply-add
+# (15 digit pairs, or 21 in the FP64 form, four real products each), at mma.sync's
+# 1,024 per clock and SM
+NEAR_FP16_MACS_PER_CMAC = 60
+NEAR_FP16_MACS_PER_CMAC_FP64 = 84
+FP16_MMA_SYNC_MACS_PER_SM = 1024
 
 
 def fp32_peak_tflops(sm_max_mhz):
@@ -70,11 +75,9 @@ def fp32_peak_tflops(sm_max_mhz):
 # DRAM bytes per launch of the class's main kernel from a one-pass ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum) of this bench command on the
 # same workload, keyed by (workload, kernel class); an entry holds only while
-# that kernel is unchanged.  near_A: the k_near_rows_df8 launch of the A part
-# (all 64 right-hand sides); translation_mac_top_tc: one top-level
+# that kernel is unchanged.  translation_mac_top_tc: one top-level
 # k_mac_top_tc2<2> launch (one chunk pair).
 NCU_DRAM_BYTES_PER_LAUNCH = {
-    ("sphere20", "near_A"): 174.58e9 + 1.26e9,
     ("sphere20", "translation_mac_top_tc"): 25.08e9 + 18.84e9,
 }
 
@@ -281,11 +284,11 @@ def run_ours(args, w, rank, world, local_rank):
         if name in ("translation_mac_top_tc", "translation_mac_tc"):
             return ("tensor", tf32_pk, f"{psrc} BF16 {bf16_kind} {bf16_pk:.1f} TFLOP/s x 1.1/2.25 "
                     f"(TF32/BF16 nominal) / {TF32_SPLIT_TERMS} split terms (FP32-accurate products)")
-        if mixed and name in ("near_A", "near_V"):
-            # double-float near field: 48 FP32 instructions per complex MAC (8 algorithmic flops)
-            return ("alu", fp32_pk / 2.0 * 8.0 / DF_INSTR_PER_CMAC,
-                    f"{n_sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x {sm_max:.0f} MHz instruction issue / "
-                    f"{DF_INSTR_PER_CMAC} FP32 instructions per double-float complex MAC x 8 flops")
+        if name in ("near_A", "near_V"):
+            macs = NEAR_FP16_MACS_PER_CMAC if mixed else NEAR_FP16_MACS_PER_CMAC_FP64
+            return ("tensor", n_sms * FP16_MMA_SYNC_MACS_PER_SM * sm_max * 1e6 / macs * 8.0 / 1e12,
+                    f"{n_sms} SMs x {FP16_MMA_SYNC_MACS_PER_SM} FP16 multiply-adds per clock (mma.sync) x {sm_max:.0f} "
+                    f"MHz / {macs} per complex MAC x 8 flops")
         if mixed:
             return ("alu", fp32_pk, f"{n_sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 flops x {sm_max:.0f} MHz")
         return ("alu", FP64_TFLOPS_NOMINAL, "NVIDIA nominal FP64 (non-tensor) rate of GB300")
@@ -332,8 +335,8 @@ def run_ours(args, w, rank, world, local_rank):
         "warmup": args.warmup, "ms_per_step": total_s * 1000.0 / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None,
         "dtype": (("c64 far (top-level translation on tensor cores: tcgen05 TF32 with a 3-term split of every FP32 "
-                   "operand) / double-float near (two FP32 words, 48-bit significand) / c128 assembly, projectors, "
-                   "Krylov") if tc_top else "c64 far / double-float near / c128 assembly, projectors, Krylov")
+                   "operand) / near field on tensor cores (double-float entries cut into 10-bit FP16 digits, 50 bits) / c128 assembly, projectors, "
+                   "Krylov") if tc_top else "c64 far / near field on tensor cores (10-bit FP16 digits, 50 bits) / c128 assembly, projectors, Krylov")
                  if mixed else "c128",
         "data": "synthetic (seeded geodesic sphere mesh, seeded complex Gaussian currents)",
         "config": {"workload": args.workload, "n_unknowns": N, "n_triangles": int(T.shape[0]),

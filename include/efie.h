@@ -381,12 +381,12 @@ int efie_precond_gradient(efie_handle *h, const void *r, const void *e, float *g
  * cores; 5: as 0 with a persistent form whose loader warp stages index
  * blocks, source spectra and kernel rows in shared memory by asynchronous
  * copies) and, for
- * mixed handles, each near-field
- * kernel (0: source values staged in shared memory by double-buffered
- * asynchronous copies, one thread per row and 8 right-hand sides; 1: read
- * through L1 with no barriers; 2: staged by the block between barriers, 4
- * right-hand sides per thread; 3: as 0 with the staging in an mbarrier ring
- * filled by a copy warp, so that row warps never wait on one another), and
+ * mixed handles, each near-field kernel (0: tensor cores, every operand cut
+ * into 10-bit digits whose FP16 products are summed exactly; 1 to 3:
+ * double-float arithmetic, with the source values 1: read through L1 with no
+ * barriers; 2: staged by the block between barriers, 4 right-hand sides per
+ * thread; 3: in an mbarrier ring filled by a copy warp, 8 right-hand sides
+ * per thread, so that row warps never wait on one another), and
  * keeps the fastest in the handle; the
  * choices are returned if the pointers are set. */
 int efie_autotune(efie_handle *h, int n_rhs, void *stream, int *best_chunk, int *best_mac, int *best_near);

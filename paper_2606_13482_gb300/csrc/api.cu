@@ -55,17 +55,48 @@ void cuda_check(cudaError_t e, const char* what) {
 struct DevMem {
   std::vector<std::pair<void*, int64_t>> ptrs;
   int64_t bytes = 0, limit = 0;
+  // buffers that only make products faster: drop() releases them, and is
+  // called where that makes room for an allocation that would fail otherwise
+  int64_t optional_bytes = 0;
+  std::function<void()> drop;
   template <typename T>
   T* alloc(int64_t n) {
     if (n <= 0) n = 1;
     int64_t b = n * (int64_t)sizeof(T);
+    if (limit > 0 && bytes + b > limit && optional_bytes > 0 && bytes - optional_bytes + b <= limit) drop();
     if (limit > 0 && bytes + b > limit)
       throw EfieError{EFIE_ENOMEM, "device_mem_limit exceeded (" + std::to_string(bytes + b) + " bytes)"};
     void* p = nullptr;
-    cuda_check(cudaMalloc(&p, (size_t)b), "cudaMalloc");
+    cudaError_t e = cudaMalloc(&p, (size_t)b);
+    if (e == cudaErrorMemoryAllocation && optional_bytes > 0) {
+      cudaGetLastError();
+      drop();
+      e = cudaMalloc(&p, (size_t)b);
+    }
+    cuda_check(e, "cudaMalloc");
     ptrs.push_back({p, b});
     bytes += b;
     return (T*)p;
+  }
+  // null where the limit or the device has no room
+  template <typename T>
+  T* alloc_optional(int64_t n) {
+    const int64_t b = std::max<int64_t>(n, 1) * (int64_t)sizeof(T);
+    if (limit > 0 && bytes + b > limit) return nullptr;
+    void* p = nullptr;
+    if (cudaMalloc(&p, (size_t)b) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    ptrs.push_back({p, b});
+    bytes += b;
+    optional_bytes += b;
+    return (T*)p;
+  }
+  void release_optional(void* p) {
+    const int64_t before = bytes;
+    release(p);
+    optional_bytes -= before - bytes;
   }
   template <typename T>
   T* upload(const std::vector<T>& v) {
@@ -280,10 +311,10 @@ struct efie_handle {
                          // interaction-list levels on CUDA cores, 5 as 0 with the loader-fed persistent form
   int* err_host = nullptr;  // host-mapped flag that device waits set when they run out
   int* err_dev = nullptr;
-  int near_variant = 0;  // mixed near field (autotuner knob): 0 x staged in shared memory by
-                         // double-buffered asynchronous copies, one thread per row and 8 RHS; 1 x
-                         // through L1; 2 x staged by the block between barriers, 4 RHS per thread;
-                         // 3 as 0 with an mbarrier ring filled by a copy warp
+  int near_variant = 0;  // mixed near field (autotuner knob): 0 tensor cores; 1 double-float, x
+                         // through L1; 2 double-float, x staged by the block between barriers, 4
+                         // RHS per thread; 3 double-float, 8 RHS per thread, x in an mbarrier ring
+                         // filled by a copy warp
   int fft_variant = 3;   // transform schedule (autotuner knob): 0 line passes; 1 forward y and z passes
                          // fused per slab where they apply (FP32, 32 channels); 2 forward and inverse
                          // fused; 3 (default) both fused on levels of 9 splines per axis only
@@ -299,6 +330,16 @@ struct efie_handle {
   float4 *xs4 = nullptr, *rho4 = nullptr;
   float2 *xsf = nullptr, *rhof = nullptr;   // FP32 copies for the far field
   bool near_df = false;   // near matrices stored as double-float pairs
+  // near field on the tensor cores (near_mma.cu): row exponents, tiles and
+  // column-group offsets of A and of the scalar part, and the digits of x for
+  // dig_ntt groups of 8 right-hand sides (optional: without them the products
+  // run on the other near kernels)
+  bool near_mma = false;
+  NearMma nmA = {}, nmS = {};
+  int64_t nkgA = 0, nkgS = 0;
+  int dig_ntt = 0;
+  // counts the (re)allocations of buffers that captured products refer to
+  int64_t buf_gen = 0;
 };
 
 namespace {
@@ -492,6 +533,7 @@ std::vector<double2*> build_kernel_spectra64(efie_handle* h, cudaStream_t s, int
 template <typename R>
 void ensure_far_buffers(efie_handle* h, FarSet<R>& F, int Rc) {
   if (F.Rc >= Rc) return;
+  ++h->buf_gen;
   Plan& P = h->plan;
   for (auto* p : F.q) h->mem.release(p);
   for (auto* p : F.r) h->mem.release(p);
@@ -526,6 +568,7 @@ void ensure_far_buffers(efie_handle* h, FarSet<R>& F, int Rc) {
 
 void ensure_work(efie_handle* h, int Rw) {
   if (h->Rw >= Rw) return;
+  ++h->buf_gen;
   for (void* p : {(void*)h->xs, (void*)h->yA, (void*)h->rho, (void*)h->w, (void*)h->xs4, (void*)h->rho4,
                   (void*)h->xsf, (void*)h->rhof, (void*)h->yAn, (void*)h->wn, (void*)h->wd})
     h->mem.release(p);
@@ -537,10 +580,7 @@ void ensure_work(efie_handle* h, int Rw) {
   h->yAn = h->mem.alloc<double2>(N * Rw);
   h->wn = h->mem.alloc<double2>(h->n_sc * Rw);
   if (h->dyadic) h->wd = h->mem.alloc<double2>(h->n_sc * Rw);
-  if (h->near_df) {
-    h->xs4 = h->mem.alloc<float4>(N * Rw);
-    h->rho4 = h->mem.alloc<float4>(Nt * Rw);
-  }
+  h->xs4 = h->rho4 = nullptr;
   if (h->precision == EFIE_MIXED) {
     h->xsf = h->mem.alloc<float2>(N * Rw);
     h->rhof = h->mem.alloc<float2>(Nt * Rw);
@@ -548,11 +588,78 @@ void ensure_work(efie_handle* h, int Rw) {
   h->Rw = Rw;
 }
 
+// double-float copies of the work vectors, for the near kernels that read them
+void ensure_split(efie_handle* h) {
+  if (h->xs4) return;
+  ++h->buf_gen;
+  h->xs4 = h->mem.alloc<float4>(h->plan.g.N * h->Rw);
+  h->rho4 = h->mem.alloc<float4>(h->plan.g.nt * h->Rw);
+}
+
+void drop_digits(efie_handle* h) {
+  if (h->dig_ntt) ++h->buf_gen;
+  h->dig_ntt = 0;
+  NearMma &A = h->nmA, &S = h->nmS;
+  if (S.xd != A.xd) {
+    h->mem.release_optional(const_cast<uint2*>(S.xd));
+    h->mem.release_optional(const_cast<int16_t*>(S.xexp));
+  }
+  h->mem.release_optional(const_cast<uint2*>(A.xd));
+  h->mem.release_optional(const_cast<int16_t*>(A.xexp));
+  A.xd = S.xd = nullptr;
+  A.xexp = S.xexp = nullptr;
+}
+
+// gives back everything that only the tensor-core near field needs; products
+// run on the other near kernels from then on
+void drop_near_mma(efie_handle* h) {
+  drop_digits(h);
+  for (NearMma* m : {&h->nmA, &h->nmS}) {
+    h->mem.release_optional(const_cast<int64_t*>(m->rexp_off));
+    h->mem.release_optional(const_cast<int64_t*>(m->kg_off));
+    h->mem.release_optional(const_cast<int32_t*>(m->tiles));
+    h->mem.release_optional(const_cast<int16_t*>(m->rexp));
+    *m = NearMma{};
+  }
+  h->near_mma = false;
+}
+
+// Whether the tensor-core near field takes nr right-hand sides on `s`, with its
+// digit buffers in place.  They are optional: where the memory limit leaves no
+// room for them, and while `s` is being captured, the products go without.
+bool ensure_digits(efie_handle* h, int nr, cudaStream_t s) {
+  if (!h->near_mma || nr > near_mma_max_nr(!h->near_df) || (h->near_df && h->near_variant != 0)) return false;
+  const int ntt = near_mma_ntiles8(nr);
+  if (h->dig_ntt >= ntt) return true;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;
+  drop_digits(h);
+  const int64_t per = 32 * (int64_t)ntt * near_mma_digits(!h->near_df), NL = h->plan.n_leaves;
+  NearMma &A = h->nmA, &S = h->nmS;
+  A.xd = h->mem.alloc_optional<uint2>(h->nkgA * per);
+  A.xexp = A.xd ? h->mem.alloc_optional<int16_t>(NL * 8 * ntt) : nullptr;
+  if (h->direct) {
+    S.xd = A.xd;
+    S.xexp = A.xexp;
+  } else if (A.xexp) {
+    S.xd = h->mem.alloc_optional<uint2>(h->nkgS * per);
+    S.xexp = S.xd ? h->mem.alloc_optional<int16_t>(NL * 8 * ntt) : nullptr;
+  }
+  if (!S.xexp) {
+    drop_digits(h);
+    return false;
+  }
+  ++h->buf_gen;
+  h->dig_ntt = ntt;
+  return true;
+}
+
 // buffers of the second chunk of a pair (FP32 far field, 8 right-hand sides):
 // its level grids q2[], r2[], and spectra buffers of the size of the largest
 // level (Qt2 for its sources, Rt2 for its results)
 void ensure_pair_buffers(efie_handle* h, FarSet<float>& F) {
   if (F.Qt2) return;
+  ++h->buf_gen;
   Plan& P = h->plan;
   const int64_t C = 32;
   F.q2.assign(P.lv.size(), nullptr);
@@ -705,6 +812,7 @@ void inv_level(efie_handle* h, FarSet<R>& F, int ell, int C, const cpx_t<R>* Rin
 template <typename R>
 void ensure_dyad_buffers(efie_handle* h, FarSet<R>& F, int Rc) {
   if (F.Rd >= Rc) return;
+  ++h->buf_gen;
   Plan& P = h->plan;
   for (auto* p : F.rd) h->mem.release(p);
   if (F.Rdh) h->mem.release(F.Rdh);
@@ -866,12 +974,43 @@ void near_fork(efie_handle* h, int nr, cudaStream_t s) {
   const int64_t N = P.g.N, Nt = P.g.nt;
   const int64_t BD = P.n_leaves;
   cudaStream_t sn = h->s_near;
+  const bool mma = ensure_digits(h, nr, s);
+  if (!mma && h->near_df) ensure_split(h);
   cuda_check(cudaEventRecord(h->ev_fork, s), "near fork");
   cuda_check(cudaStreamWaitEvent(sn, h->ev_fork, 0), "near fork");
   cuda_check(cudaStreamWaitEvent(h->s_far, h->ev_fork, 0), "far fork");
-  cuda_check(cudaMemsetAsync(h->yAn, 0, sizeof(double2) * N * nr, sn), "near outputs");
-  cuda_check(cudaMemsetAsync(h->wn, 0, sizeof(double2) * h->n_sc * nr, sn), "near outputs");
-  if (h->near_df) {
+  if (!mma) {  // these kernels add to their outputs; the tensor-core form writes every row
+    cuda_check(cudaMemsetAsync(h->yAn, 0, sizeof(double2) * N * nr, sn), "near outputs");
+    cuda_check(cudaMemsetAsync(h->wn, 0, sizeof(double2) * h->n_sc * nr, sn), "near outputs");
+  }
+  if (mma) {
+    // A and the scalar part (V on the charges, or Phi on the currents) in one
+    // launch, so that the second fills the first one's last wave; apart while
+    // kernel classes are being timed
+    NearMma A = h->nmA, S = h->nmS, none = {};
+    A.y = h->yAn;
+    A.ld = N;
+    S.y = h->wn;
+    S.ld = h->n_sc;
+    const bool f64 = !h->near_df;
+    const bool apart = h->prof.on;
+    {
+      KScope ks(h, K_NEAR_A, sn, apart || h->direct ? 2 : 3);
+      launch_near_digits(h->xs, N, nr, f64, A.box_ptr, BD, A.kg_off, const_cast<uint2*>(A.xd),
+                         const_cast<int16_t*>(A.xexp), sn);
+      if (!apart && !h->direct)
+        launch_near_digits(h->rho, Nt, nr, f64, S.box_ptr, BD, S.kg_off, const_cast<uint2*>(S.xd),
+                           const_cast<int16_t*>(S.xexp), sn);
+      launch_near_mma(A, apart ? none : S, nr, f64, sn);
+    }
+    if (apart) {
+      KScope ks(h, K_NEAR_V, sn, h->direct ? 1 : 2);
+      if (!h->direct)
+        launch_near_digits(h->rho, Nt, nr, f64, S.box_ptr, BD, S.kg_off, const_cast<uint2*>(S.xd),
+                           const_cast<int16_t*>(S.xexp), sn);
+      launch_near_mma(S, none, nr, f64, sn);
+    }
+  } else if (h->near_df) {
     {
       KScope ks(h, K_NEAR_A, sn, 2);
       launch_split_vec(h->xs, h->xs4, N * nr, sn);
@@ -1498,6 +1637,52 @@ void setup_impl(efie_handle* h, const efie_mesh* mesh, double k, int p, double g
       cuda_check(cudaStreamSynchronize(s), "near split");
       h->near_df = true;
     }
+    // tables of the tensor-core near field; without room for them the products
+    // run on the other near kernels
+    M.drop = [h] { drop_near_mma(h); };
+    bool room = true;
+    const auto up = [&](const auto& v) {
+      using T = typename std::decay<decltype(v[0])>::type;
+      T* d = room ? M.alloc_optional<T>((int64_t)v.size()) : nullptr;
+      room = room && d;
+      if (d && !v.empty())
+        cuda_check(cudaMemcpy(d, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice), "near tables");
+      return d;
+    };
+    const auto tables = [&](NearMma& m, const double2* E, const int64_t* blk_off, const std::vector<int64_t>& bp,
+                            const int64_t* d_bp, int64_t& nkg) {
+      std::vector<int64_t> roff(BD + 1, 0), kg(BD + 1, 0);
+      std::vector<int32_t> tiles;
+      for (int64_t x = 0; x < BD; ++x) {
+        const int64_t nr = bp[x + 1] - bp[x];
+        roff[x + 1] = roff[x] + (P.near_ptr[x + 1] - P.near_ptr[x]) * nr;
+        kg[x + 1] = kg[x] + (nr + 7) / 8;
+        for (int64_t r = 0; r < nr; r += NEAR_MMA_ROWS) {
+          tiles.push_back((int32_t)x);
+          tiles.push_back((int32_t)r);
+        }
+      }
+      nkg = kg[BD];
+      m.M = E;
+      m.blk_off = blk_off;
+      m.near_ptr = h->d_near_ptr;
+      m.near_src = h->d_near_src;
+      m.box_ptr = d_bp;
+      m.rexp_off = up(roff);
+      m.kg_off = up(kg);
+      m.tiles = up(tiles);
+      m.ntiles = (int)(tiles.size() / 2);
+      int16_t* rx = room ? M.alloc_optional<int16_t>(roff[BD]) : nullptr;
+      room = room && rx;
+      m.rexp = rx;
+      if (room)
+        launch_near_rexp(E, !h->near_df, blk_off, h->d_near_ptr, h->d_near_src, nd.blk_tgt, nblk, d_bp, m.rexp_off,
+                         rx, s);
+    };
+    tables(h->nmA, nd.A, h->d_blkA_off, P.box_rwg_ptr, h->d_box_rwg_ptr, h->nkgA);
+    tables(h->nmS, nd.Vn, h->d_blkS_off, h->direct ? P.box_rwg_ptr : P.box_tri_ptr, h->d_sc_box_ptr, h->nkgS);
+    h->near_mma = room;
+    if (!room) drop_near_mma(h);
   }
   cuda_check(cudaStreamSynchronize(s), "near setup");
   phase_done(2);
@@ -2699,6 +2884,7 @@ struct efie_batch {
   std::vector<const void*> key_x;
   std::vector<void*> key_y;
   std::vector<int> key_n;
+  std::vector<int64_t> key_gen;  // the members' buffer generations at capture
   int64_t launches = 0;
   std::string err;
   ~efie_batch() {
@@ -2756,7 +2942,13 @@ int efie_batch_matvec(efie_batch* b, const void* const* x, void* const* y, const
     for (size_t i = 0; i < n; ++i)
       if (kn[i] < 0 || (kn[i] > 0 && (!x[i] || !y[i] || x[i] == y[i])))
         throw EfieError{EFIE_EINVAL, "bad batch arguments (member " + std::to_string(i) + ")"};
-    if (!b->exec || kx != b->key_x || ky != b->key_y || kn != b->key_n) {
+    // buffers that a member has given back or grown since the capture
+    const auto gens = [&] {
+      std::vector<int64_t> g(n);
+      for (size_t i = 0; i < n; ++i) g[i] = b->hs[i]->buf_gen;
+      return g;
+    };
+    if (!b->exec || kx != b->key_x || ky != b->key_y || kn != b->key_n || gens() != b->key_gen) {
       // allocate every member's buffers outside the capture
       for (size_t i = 0; i < n; ++i) {
         efie_handle* h = b->hs[i];
@@ -2792,6 +2984,7 @@ int efie_batch_matvec(efie_batch* b, const void* const* x, void* const* y, const
       b->key_x = kx;
       b->key_y = ky;
       b->key_n = kn;
+      b->key_gen = gens();
     }
     cuda_check(cudaGraphLaunch(b->exec, s), "graph launch");
     b->launches++;

@@ -66,6 +66,36 @@ void launch_near_spmv_df(const float4* M, const int64_t* blk_off, const int64_t*
                          const int32_t* near_src, const int64_t* box_ptr, int64_t n_boxes, const float4* x,
                          double2* y, int64_t ld, int nr, int variant, int* err, cudaStream_t s);
 
+// Near-field product on the tensor cores (near_mma.cu): one near operator (A,
+// or the scalar part) in the layout of NearDev, with the exponents of its block
+// rows, the digits of its x, and its list of (box, first row) tiles.
+struct NearMma {
+  const void* M;             // double2 entries, or float4 double-float pairs
+  const int64_t* blk_off;
+  const int64_t* near_ptr;
+  const int32_t* near_src;
+  const int64_t* box_ptr;
+  const int64_t* rexp_off;   // [boxes] first row exponent of the box's blocks
+  const int16_t* rexp;       // [blocks of the box][rows]
+  const int64_t* kg_off;     // [boxes] first group of 8 columns of the box
+  const uint2* xd;
+  const int16_t* xexp;       // [boxes][8 ntiles8]
+  const int32_t* tiles;      // [ntiles][2]
+  int ntiles;
+  double2* y;
+  int64_t ld;
+};
+constexpr int NEAR_MMA_ROWS = 16;   // rows per tile
+int near_mma_max_nr(bool f64);      // right-hand sides that one launch takes
+int near_mma_ntiles8(int nr);       // groups of 8 right-hand sides that the digits are laid out for
+int near_mma_digits(bool f64);      // digits per value (4 bytes per digit and complex value)
+void launch_near_rexp(const void* M, bool f64, const int64_t* blk_off, const int64_t* near_ptr,
+                      const int32_t* near_src, const int32_t* blk_tgt, int64_t n_blocks, const int64_t* box_ptr,
+                      const int64_t* rexp_off, int16_t* rexp, cudaStream_t s);
+void launch_near_digits(const double2* x, int64_t ld, int nr, bool f64, const int64_t* box_ptr, int64_t n_boxes,
+                        const int64_t* kg_off, uint2* xd, int16_t* xexp, cudaStream_t s);
+void launch_near_mma(const NearMma& a, const NearMma& b, int nr, bool f64, cudaStream_t s);
+
 // Strided tensor view of a box-batched 3D grid with channels innermost:
 // element (b, i0, i1, i2, c) at b*sb + i0*s0 + i1*s1 + i2*s2 + c.
 struct View {
