@@ -18,6 +18,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "device_api.cuh"
@@ -175,7 +176,7 @@ static bool dispatch_mode_line(const cpx_t<R>* in, View vin, cpx_t<R>* out, View
   const bool two = (C % 2) == 0 && sizeof(R) == 4;
 #define EFIE_ML(NM)                                                                                          \
   if (nin <= NM) {                                                                                           \
-    if constexpr (sizeof(R) == 4 && NM <= 21) {                                                              \
+    if constexpr (sizeof(R) == 4) {                                                                          \
       if (two) {                                                                                             \
         run_mode_line<R, CM, NM, 2>(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M0, M1, sel, srcmap,     \
                                     accumulate, smem, s);                                                    \
@@ -189,9 +190,262 @@ static bool dispatch_mode_line(const cpx_t<R>* in, View vin, cpx_t<R>* out, View
   EFIE_ML(9)
   EFIE_ML(13)
   EFIE_ML(21)
-  EFIE_ML(40)
 #undef EFIE_ML
   return false;
+}
+
+// ---------------------------------------------------------------- tiled mode products
+// Mode products along long axes (more than 21 splines in, or more than 40
+// values): a small GEMM per group of 32 lines-of-16-bytes.  A block holds the
+// matrix in shared memory for all of its groups, transposed to [in][out] and cut
+// into tiles of 8 outputs; the group's input lines are staged by double-buffered
+// 16-byte asynchronous copies; a warp owns JT outputs of all 32 units (a unit
+// is two adjacent FP32 channels or one FP64 one), so one staged input value
+// feeds JT outputs and one broadcast matrix value two (FP32) lines.
+//   MODE 0: real matrix (M1 where sel says so), 1: complex, 2: rows f and n - f of
+//   the forward transform from four real sums, 3: two sources, real (sibling-
+//   shared upward transfer).
+// Every output sums over its inputs in ascending order with the line kernels'
+// sequence of multiply-adds, so the results are theirs bit for bit.
+//
+// What bounds it: the FP32 (or FP64) multiply-adds, 4 per complex product; shared
+// memory takes 8 wavefronts for every 64 of them.  It replaces one thread per
+// output, which read every input nout times and every matrix value from L1 (k_mode),
+// and register-resident lines of up to 40 values, which spilled.  On a nonuniform
+// tree with 32 boxes of 41^3 splines (77 frequencies per axis) and 52 of 25^3, 64
+// vectors, ms: forward 333 -> 69, inverse 437 -> 69, upward 181 -> 11, downward
+// 27 -> 7.  Up to 21 inputs the register-resident line kernels stay: there the
+// passes run near the memory bandwidth.
+template <int MODE>
+struct TileArgs {
+  View vin, vout;
+  int64_t items;   // groups over all boxes
+  int ngrp;        // groups per box
+  int C, ax, nin, nout, ea, eb, n;
+  const void *M0, *M1;
+  const int8_t* sel;
+  const int64_t* srcmap;
+  bool accumulate;
+  const int64_t *src0, *src1;
+  const int8_t *bit0, *bit1;
+};
+
+__device__ __forceinline__ void tile_cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+template <typename R, int MODE, int JT>
+__global__ void __launch_bounds__(320) k_mode_tile(const cpx_t<R>* __restrict__ in, cpx_t<R>* __restrict__ out,
+                                                   const TileArgs<MODE> a) {
+  using T = cpx_t<R>;
+  constexpr int LPT = 16 / (int)sizeof(T);      // channels per unit
+  constexpr bool CM = MODE == 1 || MODE == 2;
+  using E = typename std::conditional<CM, T, R>::type;
+  constexpr int NSRC = MODE == 3 ? 2 : 1;
+  extern __shared__ __align__(16) unsigned char tile_smem[];
+  const int nj = MODE == 2 ? a.n / 2 + 1 : a.nout;
+  const int njt = (nj + JT - 1) / JT;
+  const int nmat = (MODE == 0 && a.M1 && a.M1 != a.M0) || MODE == 3 ? 2 : 1;
+  const int msz = a.nin * njt * 8;
+  E* Ms = reinterpret_cast<E*>(tile_smem);                                          // [nmat][nin][njt][8]
+  uint4* tl = reinterpret_cast<uint4*>(tile_smem + sizeof(E) * (size_t)msz * nmat); // [2][NSRC][nin][32]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+  for (int e = tid; e < msz * nmat; e += blockDim.x) {
+    const int m = e / msz, r = e - m * msz, i = r / (njt * 8), q = r - i * (njt * 8), jt = q >> 3, jl = q & 7;
+    const int j = jt * JT + jl;
+    E v = E();
+    if (jl < JT && j < nj) v = reinterpret_cast<const E*>(m ? a.M1 : a.M0)[(int64_t)j * a.nin + i];
+    Ms[e] = v;
+  }
+  const int CL = a.C / LPT;
+  const int units = a.ea * a.eb * CL;
+  const int64_t sa_in = a.ax == 0 ? a.vin.s1 : a.vin.s0, sb_in = a.ax == 2 ? a.vin.s1 : a.vin.s2;
+  const int64_t sa_out = a.ax == 0 ? a.vout.s1 : a.vout.s0, sb_out = a.ax == 2 ? a.vout.s1 : a.vout.s2;
+  const int64_t step_in = a.ax == 0 ? a.vin.s0 : (a.ax == 1 ? a.vin.s1 : a.vin.s2);
+  const int64_t step_out = a.ax == 0 ? a.vout.s0 : (a.ax == 1 ? a.vout.s1 : a.vout.s2);
+  // offset of this lane's unit inside a box
+  auto where = [&](int64_t item, int64_t& b, int& c, int& ia, int& ib) {
+    b = item / a.ngrp;
+    int u = (int)(item - b * a.ngrp) * 32 + lane;
+    const bool ok = u < units;
+    if (!ok) u = 0;
+    c = (u % CL) * LPT;
+    const int t = u / CL;
+    ib = t % a.eb;
+    ia = t / a.eb;
+    return ok;
+  };
+  auto stage = [&](int64_t item, int buf) {
+    int64_t b;
+    int c, ia, ib;
+    const bool ok = where(item, b, c, ia, ib);
+    if (ok)
+#pragma unroll
+      for (int q = 0; q < NSRC; ++q) {
+        const int64_t bs = MODE == 3 ? (q ? a.src1[b] : a.src0[b]) : a.srcmap ? a.srcmap[b] : b;
+        if (bs < 0) continue;
+        const T* ip = in + bs * a.vin.sb + ia * sa_in + ib * sb_in + c;
+        uint4* d = tl + ((size_t)(buf * NSRC + q) * a.nin) * 32 + lane;
+        for (int i = warp; i < a.nin; i += nw) tile_cp16(d + i * 32, ip + i * step_in);
+      }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  int buf = 0;
+  int64_t item = blockIdx.x;
+  if (item < a.items) stage(item, 0);
+  for (; item < a.items; item += gridDim.x, buf ^= 1) {
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();  // this group's lines are in (and Ms, the first time); the other buffer is free
+    if (item + gridDim.x < a.items) stage(item + gridDim.x, buf ^ 1);
+    int64_t b;
+    int c, ia, ib;
+    const bool ok = where(item, b, c, ia, ib);
+    T* op = out + b * a.vout.sb + ia * sa_out + ib * sb_out + c;
+    const E* Ma = Ms;
+    const E* Mb = Ms;
+    bool have0 = true, have1 = false;
+    if (MODE == 0 && nmat == 2 && a.sel && a.sel[3 * b + a.ax]) Ma += msz;
+    if (MODE == 3) {
+      have0 = a.src0[b] >= 0, have1 = a.src1[b] >= 0;
+      if (a.bit0[b]) Ma += msz;
+      if (have1 && a.bit1[b]) Mb += msz;
+    }
+    const uint4* t0 = tl + ((size_t)buf * NSRC * a.nin) * 32 + lane;
+    const uint4* t1 = t0 + (size_t)a.nin * 32;
+    for (int jt = warp; jt < njt; jt += nw) {
+      R acc[JT][MODE == 2 ? 4 * LPT : 2 * LPT];
+#pragma unroll
+      for (int j = 0; j < JT; ++j)
+#pragma unroll
+        for (int q = 0; q < (MODE == 2 ? 4 * LPT : 2 * LPT); ++q) acc[j][q] = (R)0;
+      auto run = [&](const uint4* tp, const E* M) {
+        const E* m0 = M + jt * 8;
+#pragma unroll 2
+        for (int i = 0; i < a.nin; ++i) {
+          const uint4 w = tp[i * 32];
+          T v[LPT];
+          if constexpr (LPT == 2) {
+            v[0] = mk<R>((R)__uint_as_float(w.x), (R)__uint_as_float(w.y));
+            v[1] = mk<R>((R)__uint_as_float(w.z), (R)__uint_as_float(w.w));
+          } else {
+            v[0] = mk<R>((R)__hiloint2double(w.y, w.x), (R)__hiloint2double(w.w, w.z));
+          }
+          E m[8];
+          const uint4* mp = reinterpret_cast<const uint4*>(m0 + (size_t)i * njt * 8);
+#pragma unroll
+          for (int q = 0; q < (int)sizeof(E) * 8 / 16; ++q) reinterpret_cast<uint4*>(m)[q] = mp[q];
+#pragma unroll
+          for (int j = 0; j < JT; ++j)
+#pragma unroll
+            for (int l = 0; l < LPT; ++l) {
+              if constexpr (MODE == 2) {
+                acc[j][4 * l] = fma(m[j].x, v[l].x, acc[j][4 * l]);
+                acc[j][4 * l + 1] = fma(m[j].y, v[l].y, acc[j][4 * l + 1]);
+                acc[j][4 * l + 2] = fma(m[j].x, v[l].y, acc[j][4 * l + 2]);
+                acc[j][4 * l + 3] = fma(m[j].y, v[l].x, acc[j][4 * l + 3]);
+              } else if constexpr (MODE == 1) {
+                acc[j][2 * l] = fma(m[j].x, v[l].x, acc[j][2 * l]);
+                acc[j][2 * l] = fma(-m[j].y, v[l].y, acc[j][2 * l]);
+                acc[j][2 * l + 1] = fma(m[j].x, v[l].y, acc[j][2 * l + 1]);
+                acc[j][2 * l + 1] = fma(m[j].y, v[l].x, acc[j][2 * l + 1]);
+              } else {
+                acc[j][2 * l] = fma(m[j], v[l].x, acc[j][2 * l]);
+                acc[j][2 * l + 1] = fma(m[j], v[l].y, acc[j][2 * l + 1]);
+              }
+            }
+        }
+      };
+      if constexpr (MODE == 3) {
+        if (have0 && !have1) run(t0, Ma);
+        else if (have0) {
+          // both sources of an input index before the next index
+          const E *ma = Ma + jt * 8, *mb = Mb + jt * 8;
+#pragma unroll 2
+          for (int i = 0; i < a.nin; ++i) {
+            const uint4 w[2] = {t0[i * 32], t1[i * 32]};
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              T v[LPT];
+              if constexpr (LPT == 2) {
+                v[0] = mk<R>((R)__uint_as_float(w[q].x), (R)__uint_as_float(w[q].y));
+                v[1] = mk<R>((R)__uint_as_float(w[q].z), (R)__uint_as_float(w[q].w));
+              } else {
+                v[0] = mk<R>((R)__hiloint2double(w[q].y, w[q].x), (R)__hiloint2double(w[q].w, w[q].z));
+              }
+              E m[8];
+              const uint4* mp = reinterpret_cast<const uint4*>((q ? mb : ma) + (size_t)i * njt * 8);
+#pragma unroll
+              for (int r = 0; r < (int)sizeof(E) * 8 / 16; ++r) reinterpret_cast<uint4*>(m)[r] = mp[r];
+#pragma unroll
+              for (int j = 0; j < JT; ++j)
+#pragma unroll
+                for (int l = 0; l < LPT; ++l) {
+                  acc[j][2 * l] = fma(m[j], v[l].x, acc[j][2 * l]);
+                  acc[j][2 * l + 1] = fma(m[j], v[l].y, acc[j][2 * l + 1]);
+                }
+            }
+          }
+        }
+      } else {
+        run(t0, Ma);
+      }
+      if (ok)
+#pragma unroll
+        for (int j = 0; j < JT; ++j) {
+          const int jo = jt * JT + j;
+          if (jo >= nj) break;
+#pragma unroll
+          for (int l = 0; l < LPT; ++l) {
+            if constexpr (MODE == 2) {
+              const R s1 = acc[j][4 * l], s2 = acc[j][4 * l + 1], s3 = acc[j][4 * l + 2], s4 = acc[j][4 * l + 3];
+              op[jo * step_out + l] = mk<R>(s1 - s2, s3 + s4);
+              if (jo != 0 && 2 * jo != a.n) op[(int64_t)(a.n - jo) * step_out + l] = mk<R>(s1 + s2, s3 - s4);
+            } else {
+              T r = mk<R>(acc[j][2 * l], acc[j][2 * l + 1]);
+              if (a.accumulate) r = cadd(r, op[jo * step_out + l]);
+              op[jo * step_out + l] = r;
+            }
+          }
+        }
+    }
+  }
+}
+
+// false when the matrix and two input buffers do not fit in shared memory, or
+// when a unit's 16 bytes would not be aligned (an odd channel count in FP32)
+template <typename R, int MODE>
+static bool launch_mode_tile(const cpx_t<R>* in, cpx_t<R>* out, int64_t B, TileArgs<MODE> a, cudaStream_t s) {
+  constexpr int LPT = 16 / (int)sizeof(cpx_t<R>);
+  constexpr bool CM = MODE == 1 || MODE == 2;
+  if (a.C % LPT != 0) return false;
+  const int nj = MODE == 2 ? a.n / 2 + 1 : a.nout;
+  const int jt = ((nj + 6) / 7) * 7 < ((nj + 7) / 8) * 8 ? 7 : 8;  // the tile that leaves less of its last one empty
+  const int njt = (nj + jt - 1) / jt;
+  const int nmat = (MODE == 0 && a.M1 && a.M1 != a.M0) || MODE == 3 ? 2 : 1;
+  const size_t smem = (CM ? 2 : 1) * sizeof(R) * (size_t)a.nin * njt * 8 * nmat +
+                      (size_t)2 * (MODE == 3 ? 2 : 1) * a.nin * 512;
+  if (smem > 200 * 1024) return false;
+  const int64_t units = (int64_t)a.ea * a.eb * (a.C / LPT);
+  if (units > 0x7fffffff - 32) return false;
+  a.ngrp = (int)((units + 31) / 32);
+  a.items = B * a.ngrp;
+  if (a.items <= 0) return true;
+  // warps share the staged lines: one per output tile, at most 10
+  const int per = (njt + 9) / 10, warps = (njt + per - 1) / per;
+  int bps = (int)std::min<size_t>(220 * 1024 / (smem + 1024), 2048 / (size_t)(32 * warps));
+  bps = std::max(1, std::min(bps, 16));
+  const int64_t blocks = std::min<int64_t>(a.items, (int64_t)152 * bps);
+  if (jt == 7) {
+    static SmemAttr attr;
+    smem_attr_once(k_mode_tile<R, MODE, 7>, (int)smem, attr.v);
+    k_mode_tile<R, MODE, 7><<<(unsigned)blocks, 32 * warps, smem, s>>>(in, out, a);
+  } else {
+    static SmemAttr attr;
+    smem_attr_once(k_mode_tile<R, MODE, 8>, (int)smem, attr.v);
+    k_mode_tile<R, MODE, 8><<<(unsigned)blocks, 32 * warps, smem, s>>>(in, out, a);
+  }
+  return true;
 }
 
 // ---------------------------------------------------------------- sibling-shared transfers
@@ -306,8 +560,14 @@ void launch_mode_pair(const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, in
   EFIE_MP(9)
   EFIE_MP(13)
   EFIE_MP(21)
-  EFIE_MP(TRANSFER_MAX_SPLINES)
 #undef EFIE_MP
+  if (nin <= TRANSFER_MAX_SPLINES) {
+    TileArgs<3> t{};
+    t.vin = vin, t.vout = vout, t.C = C, t.ax = ax, t.nin = nin, t.nout = nout, t.ea = ea, t.eb = eb;
+    t.M0 = M0, t.M1 = M1, t.src0 = src0, t.src1 = src1, t.bit0 = bit0, t.bit1 = bit1;
+    if (launch_mode_tile<R, 3>(in, out, G, t, s)) return;
+    throw EfieError{EFIE_EINVAL, "transfer: the parent level has too many splines per axis"};
+  }
   throw EfieError{EFIE_EINVAL, "transfer: more than 40 splines per axis below the top level"};
 }
 
@@ -711,8 +971,8 @@ bool launch_dft(const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, int64_t 
     if (smem > 96 * 1024) return false;
 #define EFIE_DF(NM)                                                                                          \
   if (nin <= NM) {                                                                                           \
-    if (two && NM <= 21) {                                                                                   \
-      auto k = k_dft_fwd_line<R, NM, (sizeof(R) == 4 && NM <= 21) ? 2 : 1>;                                  \
+    if (two) {                                                                                               \
+      auto k = k_dft_fwd_line<R, NM, sizeof(R) == 4 ? 2 : 1>;                                                \
       static SmemAttr attr;                                                                  \
       smem_attr_once(k, 96 * 1024, attr.v);                                                                    \
       k<<<(unsigned)blocks, 128, smem, s>>>(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n);            \
@@ -730,8 +990,13 @@ bool launch_dft(const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, int64_t 
     EFIE_DF(9)
     EFIE_DF(13)
     EFIE_DF(21)
-    EFIE_DF(40)
 #undef EFIE_DF
+    if (nin <= 40) {
+      TileArgs<2> t{};
+      t.vin = vin, t.vout = vout, t.C = C, t.ax = ax, t.nin = nin, t.nout = nout, t.ea = ea, t.eb = eb, t.n = n;
+      t.M0 = M;
+      return launch_mode_tile<R, 2>(in, out, B, t, s);
+    }
     return false;
   }
   const size_t smem = sizeof(T) * (size_t)nout * nh;
@@ -776,6 +1041,18 @@ void launch_mode(const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, int64_t
                           : dispatch_mode_line<R, false>(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M0, M1,
                                                          sel, srcmap, accumulate, smem, s);
     if (done) return;
+  }
+  {
+    const int ea = ax == 0 ? e1 : e0, eb = ax == 2 ? e1 : e2;
+    const auto fill = [&](auto t) {
+      t.vin = vin, t.vout = vout, t.C = C, t.ax = ax, t.nin = nin, t.nout = nout, t.ea = ea, t.eb = eb;
+      t.M0 = M0, t.M1 = M1, t.sel = sel, t.srcmap = srcmap, t.accumulate = accumulate;
+      return t;
+    };
+    // one complex matrix (sel picks between two real ones only)
+    if (complex_m ? (M1 == nullptr || M1 == M0) && launch_mode_tile<R, 1>(in, out, B, fill(TileArgs<1>{}), s)
+                  : launch_mode_tile<R, 0>(in, out, B, fill(TileArgs<0>{}), s))
+      return;
   }
   int64_t blocks = ceil_div(total, 256);
   if (blocks > 152 * 64) blocks = 152 * 64;
