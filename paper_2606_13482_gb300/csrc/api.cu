@@ -188,6 +188,7 @@ struct LevDev {
   // gather-list offsets of their grid points
   int64_t leaf0 = 0, nleaf = 0;
   int32_t* leaf_box = nullptr;
+  int max_rwg = 0, max_sc = 0;   // functions of the largest leaf
   int32_t *gptr_r = nullptr, *gptr_t = nullptr;
 };
 
@@ -719,7 +720,7 @@ void anterp_up(efie_handle* h, FarSet<R>& F, int nr, int rhs0, std::vector<cpx_t
       rin = h->direct ? xin : (const cpx_t<R>*)(h->rhof + (int64_t)rhs0 * Nt);
     }
     launch_anterp<R>(F.gr, F.gt, LV.gptr_r, LV.gptr_t, h->mr_off, h->mt_off, h->d_box_rwg_ptr + LV.leaf0,
-                     h->d_sc_box_ptr + LV.leaf0, LV.nleaf, LV.leaf_box, xin, N, rin, h->direct ? N : Nt, nr,
+                     h->d_sc_box_ptr + LV.leaf0, LV.nleaf, LV.max_rwg, LV.max_sc, LV.leaf_box, xin, N, rin, h->direct ? N : Nt, nr,
                      qq[ell - top], L.sp, s);
   };
   anterp(D);
@@ -1359,6 +1360,12 @@ void setup_impl(efie_handle* h, const efie_mesh* mesh, double k, int p, double g
     LD.B = (int64_t)L.code.size();
     LD.leaf0 = P.level_leaf_ptr[ell - P.top];
     LD.nleaf = P.level_leaf_ptr[ell - P.top + 1] - LD.leaf0;
+    for (int64_t x = LD.leaf0; x < LD.leaf0 + LD.nleaf; ++x) {
+      const int64_t* rp = P.box_rwg_ptr.data() + x;
+      const int64_t* tp = (h->direct ? P.box_rwg_ptr : P.box_tri_ptr).data() + x;
+      LD.max_rwg = std::max<int>(LD.max_rwg, (int)(rp[1] - rp[0]));
+      LD.max_sc = std::max<int>(LD.max_sc, (int)(tp[1] - tp[0]));
+    }
     if (LD.nleaf > 0 && LD.nleaf != LD.B) {
       std::vector<int32_t> lb(LD.nleaf);
       for (int64_t x = 0; x < LD.nleaf; ++x) lb[x] = (int32_t)P.leaf_box[LD.leaf0 + x];

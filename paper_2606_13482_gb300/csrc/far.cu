@@ -1161,25 +1161,30 @@ __global__ void k_gather_build(const R* __restrict__ mr, const int32_t* __restri
 
 // ---------------------------------------------------------------- anterpolation
 // q[b][pt][d nr + r] = sum over the gather list of pt: m_d x_r[k] (d < 3) and
-// sum of m^phi rho_r[t] (d = 3).  One CTA per leaf box; the box's currents and
-// charges are staged in shared memory (AK basis functions at a time; boxes
-// with more take several passes over their sorted lists).  A warp takes four
-// grid points at a time, lane = (point, right-hand side): the eight lanes of a
-// point read the same list entry (one broadcast) and eight consecutive staged
-// values, and own their 4 output components outright -- no atomics, no
-// reductions, each moment entry read once per launch, each output written once.
-template <typename R>
-struct AnterpCfg;
-template <>
-struct AnterpCfg<float> {
-  static constexpr int AK = 256, XS = 10;  // 80-byte rows
+// sum of m^phi rho_r[t] (d = 3).  Blocks are (leaf box, part of its grid points);
+// the box's currents and charges are staged in shared memory (ak basis
+// functions at a time: all of them wherever they fit, else several passes
+// over the sorted lists).  LR lanes, the right-hand sides rounded up to a power
+// of two, share a point: a warp takes 32 / LR points at a time, the lanes of a
+// point read the same list entry (one broadcast) and consecutive staged values,
+// and own their 4 output components outright -- no atomics, no reductions,
+// each moment entry read once per launch, each output written once.
+//
+// What bounds it: the latency of the list entries, and in FP64 the multiply-
+// adds, so lanes without a right-hand side (7 of 8 with LR = 8 and one vector)
+// cost as much as the others.  One block per box left the chip empty on trees with
+// few boxes.  Measured: 1,920 unknowns, 32 boxes, FP64, one vector
+// 0.397 -> 0.078 ms; 48,000 unknowns, FP64, 8 vectors 2.75 -> 1.31 (two passes per 32
+// points before); the nonuniform tree with 22 leaves of 41^3 points on its top
+// level, 64 vectors 166 -> 5.8.
+template <typename R, int LR>
+struct AnterpCfg {
+  // values per staged function: rows of 80 bytes (FP32) and 144 (FP64) spread the banks
+  static constexpr int XS = LR < 8 ? LR : sizeof(R) == 4 ? 10 : 9;
 };
-template <>
-struct AnterpCfg<double> {
-  static constexpr int AK = 128, XS = 9;   // 144-byte rows
-};
+constexpr int ANTERP_SMEM = 96 * 1024;
 
-template <typename R>
+template <typename R, int LR>
 __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const R* __restrict__ gt,
                                                 const int32_t* __restrict__ gptr_r,
                                                 const int32_t* __restrict__ gptr_t,
@@ -1190,12 +1195,14 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
                                                 const int32_t* __restrict__ out_box,
                                                 const cpx_t<R>* __restrict__ xs, int64_t ldx,
                                                 const cpx_t<R>* __restrict__ rho, int64_t ldr, int nr,
-                                                cpx_t<R>* __restrict__ q, int sp) {
+                                                cpx_t<R>* __restrict__ q, int sp, int ak, int at, int nsplit) {
   using T = cpx_t<R>;
-  constexpr int AK = AnterpCfg<R>::AK, XS = AnterpCfg<R>::XS;
-  __shared__ __align__(16) T xsm[AK][XS];
-  __shared__ __align__(16) T rsm[AK][XS];
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int XS = AnterpCfg<R, LR>::XS, PW = 32 / LR;
+  extern __shared__ __align__(16) unsigned char anterp_smem[];
+  T* xsm = reinterpret_cast<T*>(anterp_smem);  // [ak][XS]
+  T* rsm = xsm + (size_t)ak * XS;              // [at][XS]
+  const int b = blockIdx.x / nsplit, part = blockIdx.x - b * nsplit;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int npts = sp * sp * sp;
   const int64_t k0 = box_rwg_ptr[b], t0 = box_tri_ptr[b];
   const int nk = (int)(box_rwg_ptr[b + 1] - k0), nt = (int)(box_tri_ptr[b + 1] - t0);
@@ -1203,23 +1210,28 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
   const R* get = gt + 2 * (nt > 0 ? mt_off[t0] : 0);
   const int32_t* pr = gptr_r + (int64_t)b * (npts + 1);
   const int32_t* pq = gptr_t + (int64_t)b * (npts + 1);
-  const int nchunk = max((nk + AK - 1) / AK, (nt + AK - 1) / AK);
+  const int nchunk = max((nk + ak - 1) / ak, (nt + at - 1) / at);
   auto stage = [&](int c) {
-    for (int i = tid; i < AK * nr; i += blockDim.x) {
-      const int r = i / AK, kk = i - r * AK, k = c * AK + kk;
-      if (k < nk) xsm[kk][r] = xs[r * ldx + k0 + k];
-      if (k < nt) rsm[kk][r] = rho[r * ldr + t0 + k];
+    for (int i = tid; i < ak * nr; i += blockDim.x) {
+      const int r = i / ak, kk = i - r * ak, k = c * ak + kk;
+      if (k < nk) xsm[kk * XS + r] = xs[r * ldx + k0 + k];
+    }
+    for (int i = tid; i < at * nr; i += blockDim.x) {
+      const int r = i / at, kk = i - r * at, k = c * at + kk;
+      if (k < nt) rsm[kk * XS + r] = rho[r * ldr + t0 + k];
     }
   };
   if (nchunk == 1) {
     stage(0);
     __syncthreads();
   }
-  const int r = lane & 7, ps = lane >> 3;
+  const int r = lane & (LR - 1), ps = lane / LR;
   const int C = 4 * nr;
-  const int per_pass = 4 * (blockDim.x >> 5);
-  for (int pb = 0; pb < npts; pb += per_pass) {
-    const int p = pb + 4 * warp + ps;
+  const int per_pass = PW * (blockDim.x >> 5);
+  // passes part, part + nsplit, ..: points near the surface, where the lists
+  // are long, spread over the parts
+  for (int pb = part * per_pass; pb < npts; pb += nsplit * per_pass) {
+    const int p = pb + PW * warp + ps;
     const bool okp = p < npts;
     T a0 = mk<R>(0, 0), a1 = a0, a2 = a0, a3 = a0;
     int er = okp ? pr[p] : 0, er1 = okp ? pr[p + 1] : 0;
@@ -1230,7 +1242,7 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
         stage(c);
         __syncthreads();
       }
-      const R kc0 = (R)(c * AK), kc1 = (R)((c + 1) * AK);
+      const int kc0 = c * ak, tc0 = c * at;
       auto load4 = [&](int64_t i, R& ek, R& m0, R& m1, R& m2) {
         const R* e = ger + 4 * i;
         if constexpr (sizeof(R) == 4) {
@@ -1241,8 +1253,8 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
           ek = v0.x, m0 = v0.y, m1 = v1.x, m2 = v1.y;
         }
       };
-      auto mac3 = [&](R ek, R m0, R m1, R m2) {
-        const T xv = xsm[(int)(ek - kc0)][r];
+      auto mac3 = [&](int k, R m0, R m1, R m2) {
+        const T xv = xsm[(k - kc0) * XS + r];
         a0.x = fma(m0, xv.x, a0.x);
         a0.y = fma(m0, xv.y, a0.y);
         a1.x = fma(m1, xv.x, a1.x);
@@ -1257,14 +1269,14 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
 #pragma unroll
           for (int t = 0; t < 4; ++t) load4(er + t, k_[t], x_[t], y_[t], z_[t]);
 #pragma unroll
-          for (int t = 0; t < 4; ++t) mac3(k_[t], x_[t], y_[t], z_[t]);
+          for (int t = 0; t < 4; ++t) mac3((int)k_[t], x_[t], y_[t], z_[t]);
         }
       }
       for (; er < er1; ++er) {
         R ek, m0, m1, m2;
         load4(er, ek, m0, m1, m2);
-        if (ek >= kc1) break;
-        mac3(ek, m0, m1, m2);
+        if ((int)ek >= kc0 + ak) break;
+        mac3((int)ek, m0, m1, m2);
       }
       auto load2 = [&](int64_t i, R& ek, R& m) {
         const R* e = get + 2 * i;
@@ -1276,8 +1288,8 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
           ek = v.x, m = v.y;
         }
       };
-      auto mac1 = [&](R ek, R m) {
-        const T v = rsm[(int)(ek - kc0)][r];
+      auto mac1 = [&](int k, R m) {
+        const T v = rsm[(k - tc0) * XS + r];
         a3.x = fma(m, v.x, a3.x);
         a3.y = fma(m, v.y, a3.y);
       };
@@ -1287,14 +1299,14 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
 #pragma unroll
           for (int t = 0; t < 4; ++t) load2(et + t, k_[t], m_[t]);
 #pragma unroll
-          for (int t = 0; t < 4; ++t) mac1(k_[t], m_[t]);
+          for (int t = 0; t < 4; ++t) mac1((int)k_[t], m_[t]);
         }
       }
       for (; et < et1; ++et) {
         R ek, m;
         load2(et, ek, m);
-        if (ek >= kc1) break;
-        mac1(ek, m);
+        if ((int)ek >= tc0 + at) break;
+        mac1((int)ek, m);
       }
     }
     if (okp && r < nr) {
@@ -1320,14 +1332,41 @@ void launch_gather_build(const R* mr, const int32_t* mr_base, const int32_t* mr_
                                                    box_rwg_ptr, box_tri_ptr, sp, gptr_r, gptr_t, gr, gt);
 }
 
+template <typename R, int LR>
+static void run_anterp(const R* gr, const R* gt, const int32_t* gptr_r, const int32_t* gptr_t, const int64_t* mr_off,
+                       const int64_t* mt_off, const int64_t* box_rwg_ptr, const int64_t* box_tri_ptr, int64_t B,
+                       int max_rwg, int max_sc, const int32_t* out_box, const cpx_t<R>* xs, int64_t ldx,
+                       const cpx_t<R>* rho, int64_t ldr, int nr, cpx_t<R>* q, int sp, cudaStream_t s) {
+  const size_t row = AnterpCfg<R, LR>::XS * sizeof(cpx_t<R>);
+  const int cap = (int)(ANTERP_SMEM / row);
+  int ak = std::max(1, max_rwg), at = std::max(1, max_sc);
+  if (ak + at > cap) ak = at = cap / 2;
+  const size_t smem = (size_t)(ak + at) * row;
+  static SmemAttr attr;
+  smem_attr_once(k_anterp<R, LR>, ANTERP_SMEM, attr.v);
+  // parts of a box's points, up to one pass each, until the blocks fill the
+  // chip twice over (4 blocks of 8 warps per SM); a part stages the box again
+  const int64_t npts = (int64_t)sp * sp * sp, passes = ceil_div(npts, 256 / LR);
+  const int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(passes, ceil_div(152 * 8, B)));
+  k_anterp<R, LR><<<(unsigned)(B * nsplit), 256, smem, s>>>(gr, gt, gptr_r, gptr_t, mr_off, mt_off, box_rwg_ptr,
+                                                            box_tri_ptr, out_box, xs, ldx, rho, ldr, nr, q, sp, ak, at,
+                                                            nsplit);
+}
+
 template <typename R>
 void launch_anterp(const R* gr, const R* gt, const int32_t* gptr_r, const int32_t* gptr_t, const int64_t* mr_off,
                    const int64_t* mt_off, const int64_t* box_rwg_ptr, const int64_t* box_tri_ptr, int64_t B,
-                   const int32_t* out_box, const cpx_t<R>* xs, int64_t ldx, const cpx_t<R>* rho, int64_t ldr, int nr,
-                   cpx_t<R>* q, int sp, cudaStream_t s) {
+                   int max_rwg, int max_sc, const int32_t* out_box, const cpx_t<R>* xs, int64_t ldx,
+                   const cpx_t<R>* rho, int64_t ldr, int nr, cpx_t<R>* q, int sp, cudaStream_t s) {
   if (B <= 0 || nr <= 0) return;
-  k_anterp<R><<<(unsigned)B, 256, 0, s>>>(gr, gt, gptr_r, gptr_t, mr_off, mt_off, box_rwg_ptr, box_tri_ptr, out_box,
-                                          xs, ldx, rho, ldr, nr, q, sp);
+#define EFIE_AN(L)                                                                                                   \
+  run_anterp<R, L>(gr, gt, gptr_r, gptr_t, mr_off, mt_off, box_rwg_ptr, box_tri_ptr, B, max_rwg, max_sc, out_box, xs, \
+                   ldx, rho, ldr, nr, q, sp, s)
+  if (nr == 1) EFIE_AN(1);
+  else if (nr == 2) EFIE_AN(2);
+  else if (nr <= 4) EFIE_AN(4);
+  else EFIE_AN(8);
+#undef EFIE_AN
 }
 
 // ---------------------------------------------------------------- interpolation
@@ -2256,12 +2295,11 @@ template void launch_gather_build<double>(const double*, const int32_t*, const i
                                           const int64_t*, const int64_t*, int64_t, int, int32_t*, int32_t*,
                                           double*, double*, cudaStream_t);
 template void launch_anterp<float>(const float*, const float*, const int32_t*, const int32_t*, const int64_t*,
-                                   const int64_t*, const int64_t*, const int64_t*, int64_t, const int32_t*,
+                                   const int64_t*, const int64_t*, const int64_t*, int64_t, int, int, const int32_t*,
                                    const float2*, int64_t, const float2*, int64_t, int, float2*, int, cudaStream_t);
 template void launch_anterp<double>(const double*, const double*, const int32_t*, const int32_t*, const int64_t*,
-                                    const int64_t*, const int64_t*, const int64_t*, int64_t, const int32_t*,
-                                    const double2*, int64_t, const double2*, int64_t, int, double2*, int,
-                                    cudaStream_t);
+                                    const int64_t*, const int64_t*, const int64_t*, int64_t, int, int, const int32_t*,
+                                    const double2*, int64_t, const double2*, int64_t, int, double2*, int, cudaStream_t);
 template void launch_interp<float>(const float*, const int32_t*, const int32_t*, const int64_t*, const int32_t*,
                                    int64_t, const float*, const int32_t*, const int32_t*, const int64_t*,
                                    const int32_t*, int64_t, const float2*, int, int, double2*, int64_t,
