@@ -339,6 +339,7 @@ struct efie_handle {
   NearMma nmA = {}, nmS = {};
   int64_t nkgA = 0, nkgS = 0;
   int dig_ntt = 0;
+  int max_tset = 0;       // triangles of the largest leaf's triangle set
   // counts the (re)allocations of buffers that captured products refer to
   int64_t buf_gen = 0;
 };
@@ -1548,6 +1549,7 @@ void setup_impl(efie_handle* h, const efie_mesh* mesh, double k, int p, double g
     nd.tri_perm = M.upload(P.tri_perm);
     nd.tset_ptr = M.upload(P.tset_ptr);
     nd.tset = M.upload(P.tset);
+    for (int64_t x = 0; x < BD; ++x) h->max_tset = std::max<int>(h->max_tset, (int)(P.tset_ptr[x + 1] - P.tset_ptr[x]));
     nd.rwg_tl = M.upload(P.rwg_tl);
     nd.rwg_loc = M.upload(P.rwg_loc);
     nd.rwg_coef = M.upload(P.rwg_coef);
@@ -2096,17 +2098,12 @@ bool read_weights(const char* path, std::vector<float>& p) {
 }  // namespace
 
 namespace efie {
-int handle_rhs_args(const efie_handle* h, const double** V, const int32_t** T, const double** area,
-                    const int32_t** tri_pm, const int32_t** free_pm, int64_t* N, double* k, int* device) {
+int handle_rhs_args(const efie_handle* h, RhsGeom* g, int* device) {
   if (!h) return EFIE_EINVAL;
   *device = h->device;
-  *V = h->dV;
-  *T = h->dT;
-  *area = h->darea;
-  *tri_pm = h->dtri_pm;
-  *free_pm = h->dfree_pm;
-  *N = h->plan.g.N;
-  *k = h->plan.k;
+  const NearDev& nd = h->nd;
+  *g = RhsGeom{h->dV, h->dT, h->darea, h->dtri_pm, h->dfree_pm, h->plan.g.N, h->plan.k, h->plan.n_leaves,
+               h->d_box_rwg_ptr, nd.tset_ptr, nd.tset, nd.rwg_tl, h->d_rwg_perm, h->max_tset};
   return EFIE_OK;
 }
 void handle_set_error(efie_handle* h, const char* msg) {
@@ -2419,8 +2416,10 @@ int efie_rhs_planewave(efie_handle* h, int n_rhs, const double* khat, const doub
     double* dp = h->mem.alloc<double>(3 * n_rhs);
     cuda_check(cudaMemcpyAsync(dk, khat, sizeof(double) * 3 * n_rhs, cudaMemcpyHostToDevice, s), "khat");
     cuda_check(cudaMemcpyAsync(dp, pol, sizeof(double) * 3 * n_rhs, cudaMemcpyHostToDevice, s), "pol");
-    launch_rhs_planewave(h->dV, h->dT, h->darea, h->dtri_pm, h->dfree_pm, h->plan.g.N, h->plan.k, dk, dp, n_rhs,
-                         (double2*)rhs, h->plan.g.N, s);
+    RhsGeom g;
+    int dev;
+    handle_rhs_args(h, &g, &dev);
+    launch_rhs_planewave(g, dk, dp, n_rhs, (double2*)rhs, h->plan.g.N, s);
     cuda_check(cudaStreamSynchronize(s), "rhs");
     h->mem.release(dk);
     h->mem.release(dp);

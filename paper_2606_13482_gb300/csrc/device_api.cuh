@@ -214,9 +214,22 @@ void launch_combine(const double2* yA, int64_t ldA, const double2* w, int64_t ld
                     const double2* wn, const int32_t* rwg_perm, const int32_t* rwg_tri_sorted, int64_t N, int nr,
                     double2 cA, double2 cV, double2* y, int64_t ldy, double2* yAout,
                     double2* yVout, cudaStream_t s);
-void launch_rhs_planewave(const double* V, const int32_t* T, const double* area, const int32_t* tri_pm,
-                          const int32_t* free_pm, int64_t N, double k, const double* khat,
-                          const double* pol, int nr, double2* rhs, int64_t ld, cudaStream_t s);
+// Geometry of the plane-wave right-hand sides: the mesh, and the leaf boxes
+// with their triangle sets (the triangles of each box's RWGs).
+struct RhsGeom {
+  const double* V;
+  const int32_t* T;
+  const double* area;
+  const int32_t *tri_pm, *free_pm;
+  int64_t N;
+  double k;
+  int64_t n_boxes;
+  const int64_t *box_rwg_ptr, *tset_ptr;
+  const int32_t *tset, *rwg_tl, *rwg_perm;
+  int max_tset;
+};
+void launch_rhs_planewave(const RhsGeom& g, const double* khat, const double* pol, int nr, double2* rhs, int64_t ld,
+                          cudaStream_t s);
 
 // Krylov helpers (FP64)
 void launch_multidot(const double2* Vb, int64_t ldv_r, int64_t ldv_i, int nbasis, const double2* w,

@@ -18,6 +18,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "common.cuh"
@@ -2097,7 +2098,8 @@ void launch_combine(const double2* yA, int64_t ldA, const double2* w, int64_t ld
                                              y, ldy, yAout, yVout);
 }
 
-// Plane-wave RHS: per RWG, both triangles with a degree-10 collapsed rule.
+// Plane-wave RHS: per RWG, both triangles with a degree-10 collapsed rule
+// (boxes with more than 1,472 triangles).
 __constant__ double c_q6[3][36];
 __global__ void k_rhs_pw(const double* __restrict__ V, const int32_t* __restrict__ T,
                          const double* __restrict__ area, const int32_t* __restrict__ tri_pm,
@@ -2135,17 +2137,163 @@ __global__ void k_rhs_pw(const double* __restrict__ V, const int32_t* __restrict
     rhs[r * ld + m] = acc;
   }
 }
-int upload_rhs_rule(const double* q6) {
-  return cudaMemcpyToSymbol(c_q6, q6, sizeof(double) * 108) == cudaSuccess ? 0 : -1;
+// Plane waves by leaf box: the triangles of the box's RWGs (its triangle set)
+// are integrated once per wave and combined into the RWGs, instead of 72 sines and
+// cosines per RWG.  For one triangle and wave, with x = c + (xi - 1/3) e1 +
+// (eta - 1/3) e2 (c the centroid), alpha = -k khat.e1 and beta = -k khat.e2, the points
+// of the collapsed 6 x 6 rule, xi = u_a, eta = (1 - u_a)(1/2 +- t_b), have the phases
+//   phi_c + psi_a +- t_b gamma_a,  psi_a = (u_a - 1/3)(alpha - beta / 2),  gamma_a = (1 - u_a) beta,
+// so a row a of six points needs one complex exponential of psi_a and the
+// rule's even and odd sums C = sum_b w_b cos(t_b gamma), S = sum_b w_b t_b sin(t_b gamma),
+// which are power series in gamma^2 with fixed coefficients.  Elements are a
+// fraction of a wavelength, so Taylor series of eight terms leave less than
+// 3e-16 for |gamma| <= 1 and |psi| <= 0.6; beyond (elements above lambda / 7) the row
+// calls cos and sin.  Same rule, same points as k_rhs_pw, up to rounding.
+//
+// What bounds it: the FP64 pipe, about 350 operations per triangle and wave (2 per
+// clock and SM).  38,720 triangles, 360 waves: 126 -> 12.0 ms.
+__constant__ double c_pw_u[6], c_pw_w[6], c_pw_t[3], c_pw_v[3], c_pw_c[8], c_pw_s[8];
+
+__device__ __forceinline__ double pw_poly8(const double* c, double x) {
+  double r = c[7];
+#pragma unroll
+  for (int n = 6; n >= 0; --n) r = fma(r, x, c[n]);
+  return r;
 }
-void launch_rhs_planewave(const double* V, const int32_t* T, const double* area, const int32_t* tri_pm,
-                          const int32_t* free_pm, int64_t N, double k, const double* khat,
-                          const double* pol, int nr, double2* rhs, int64_t ld, cudaStream_t s) {
-  int64_t total = N * nr;
+__global__ void __launch_bounds__(128) k_rhs_box(const RhsGeom g, const double* __restrict__ khat,
+                                                 const double* __restrict__ pol, int nr, int W,
+                                                 double2* __restrict__ rhs, int64_t ld) {
+  extern __shared__ double2 pw_smem[];  // [triangle][wave][F0, G1]
+  const int64_t t0 = g.tset_ptr[blockIdx.x], i0 = g.box_rwg_ptr[blockIdx.x];
+  const int ntri = (int)(g.tset_ptr[blockIdx.x + 1] - t0), nrwg = (int)(g.box_rwg_ptr[blockIdx.x + 1] - i0);
+  const int r0 = blockIdx.y * W, nw = min(W, nr - r0);
+  const double third = 1.0 / 3.0;
+  // Taylor coefficients of cos and sin(x) / x in x^2
+  const double tc[8] = {1.0, -1.0 / 2, 1.0 / 24, -1.0 / 720, 1.0 / 40320, -1.0 / 3628800, 1.0 / 479001600,
+                        -1.0 / 87178291200.0};
+  const double ts[8] = {1.0, -1.0 / 6, 1.0 / 120, -1.0 / 5040, 1.0 / 362880, -1.0 / 39916800, 1.0 / 6227020800.0,
+                        -1.0 / 1307674368000.0};
+  for (int e = threadIdx.x; e < ntri * nw; e += blockDim.x) {
+    const int w = e / ntri, t = e - w * ntri, tri = g.tset[t0 + t];
+    const double* kh = khat + 3 * (r0 + w);
+    const double* pl = pol + 3 * (r0 + w);
+    const double* va = g.V + 3 * (int64_t)g.T[3 * tri];
+    const double* vb = g.V + 3 * (int64_t)g.T[3 * tri + 1];
+    const double* vc = g.V + 3 * (int64_t)g.T[3 * tri + 2];
+    double phi = 0, alpha = 0, beta = 0, p1 = 0, p2 = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const double a = va[d], e1 = vb[d] - a, e2 = vc[d] - a;
+      phi = fma(kh[d], a + third * (e1 + e2), phi);
+      alpha = fma(kh[d], e1, alpha);
+      beta = fma(kh[d], e2, beta);
+      p1 = fma(pl[d], e1, p1);
+      p2 = fma(pl[d], e2, p2);
+    }
+    phi *= -g.k, alpha *= -g.k, beta *= -g.k;
+    const double delta = alpha - 0.5 * beta;
+    const bool series = fabs(beta) <= 1.0 && fabs(delta) <= 0.9;
+    double2 F0 = make_double2(0, 0), Fx = F0, Fe = F0;
+#pragma unroll 1
+    for (int a = 0; a < 6; ++a) {
+      const double u = c_pw_u[a], gam = (1.0 - u) * beta, psi = (u - third) * delta;
+      double C, S, cs, sn;
+      if (series) {
+        const double g2 = gam * gam, q2 = psi * psi;
+        C = pw_poly8(c_pw_c, g2);
+        S = gam * pw_poly8(c_pw_s, g2);
+        cs = pw_poly8(tc, q2);
+        sn = psi * pw_poly8(ts, q2);
+      } else {
+        C = S = 0;
+        for (int b = 0; b < 3; ++b) {
+          double sb, cb;
+          sincos(c_pw_t[b] * gam, &sb, &cb);
+          C = fma(c_pw_v[b], cb, C);
+          S = fma(c_pw_v[b] * c_pw_t[b], sb, S);
+        }
+        sincos(psi, &sn, &cs);
+      }
+      const double wa = c_pw_w[a], wc = wa * C, we = wa * (1.0 - u), p = 0.5 * we * C, q = we * S;
+      F0.x = fma(wc, cs, F0.x);
+      F0.y = fma(wc, sn, F0.y);
+      Fx.x = fma(u * wc, cs, Fx.x);
+      Fx.y = fma(u * wc, sn, Fx.y);
+      Fe.x = fma(p, cs, fma(-q, sn, Fe.x));
+      Fe.y = fma(p, sn, fma(q, cs, Fe.y));
+    }
+    double sp, cp;
+    sincos(phi, &sp, &cp);
+    const double2 G = make_double2(p1 * Fx.x + p2 * Fe.x, p1 * Fx.y + p2 * Fe.y);
+    pw_smem[2 * (t * W + w)] = make_double2(F0.x * cp - F0.y * sp, F0.x * sp + F0.y * cp);
+    pw_smem[2 * (t * W + w) + 1] = make_double2(G.x * cp - G.y * sp, G.x * sp + G.y * cp);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nrwg * nw; e += blockDim.x) {
+    const int w = e / nrwg, i = e - w * nrwg;
+    const int64_t m = g.rwg_perm[i0 + i];
+    const double* pl = pol + 3 * (r0 + w);
+    double2 acc = make_double2(0, 0);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int t = g.rwg_tl[2 * (i0 + i) + s];
+      const double* a = g.V + 3 * (int64_t)g.T[3 * g.tset[t0 + t]];
+      const double* xf = g.V + 3 * (int64_t)g.free_pm[2 * m + s];
+      const double d = (a[0] - xf[0]) * pl[0] + (a[1] - xf[1]) * pl[1] + (a[2] - xf[2]) * pl[2];
+      const double2 F0 = pw_smem[2 * (t * W + w)], G = pw_smem[2 * (t * W + w) + 1];
+      const double2 v = make_double2(fma(d, F0.x, G.x), fma(d, F0.y, G.y));
+      acc = s == 0 ? v : csub(acc, v);
+    }
+    rhs[(int64_t)(r0 + w) * ld + m] = acc;
+  }
+}
+int upload_rhs_rule(const double* q6) {
+  // rows of the collapsed rule: xi = u_a, eta = (1 - u_a) v_b, weight w_a v_b-weight;
+  // v_b = 1/2 -+ t_b in pairs of equal weight
+  double u[6], w[6], t[3], v[3], c[8], sc[8];
+  for (int a = 0; a < 6; ++a) {
+    u[a] = q6[6 * a];
+    w[a] = 0;
+    for (int b = 0; b < 6; ++b) w[a] += q6[72 + 6 * a + b];
+  }
+  for (int b = 0; b < 3; ++b) {
+    t[b] = q6[36 + 3 + b] / (1.0 - u[0]) - 0.5;
+    v[b] = 2.0 * q6[72 + 3 + b] / w[0];
+  }
+  double fc = 1.0, fs = 1.0;  // (2n)!, (2n + 1)! with the sign
+  for (int n = 0; n < 8; ++n) {
+    if (n) fc *= -(2.0 * n) * (2.0 * n - 1.0), fs *= -(2.0 * n) * (2.0 * n + 1.0);
+    c[n] = sc[n] = 0;
+    for (int b = 0; b < 3; ++b) {
+      c[n] += v[b] * std::pow(t[b], 2 * n) / fc;
+      sc[n] += v[b] * std::pow(t[b], 2 * n + 2) / fs;
+    }
+  }
+  const bool ok = cudaMemcpyToSymbol(c_q6, q6, sizeof(double) * 108) == cudaSuccess &&
+                  cudaMemcpyToSymbol(c_pw_u, u, sizeof(u)) == cudaSuccess &&
+                  cudaMemcpyToSymbol(c_pw_w, w, sizeof(w)) == cudaSuccess &&
+                  cudaMemcpyToSymbol(c_pw_t, t, sizeof(t)) == cudaSuccess &&
+                  cudaMemcpyToSymbol(c_pw_v, v, sizeof(v)) == cudaSuccess &&
+                  cudaMemcpyToSymbol(c_pw_c, c, sizeof(c)) == cudaSuccess &&
+                  cudaMemcpyToSymbol(c_pw_s, sc, sizeof(sc)) == cudaSuccess;
+  return ok ? 0 : -1;
+}
+void launch_rhs_planewave(const RhsGeom& g, const double* khat, const double* pol, int nr, double2* rhs, int64_t ld,
+                          cudaStream_t s) {
+  int64_t total = g.N * nr;
   if (total <= 0) return;
+  // by leaf box where its triangles' integrals fit in shared memory, up to 8
+  // waves at a time (46 KB: no opt-in, four blocks per SM)
+  const int64_t per = 2 * sizeof(double2) * (int64_t)g.max_tset;
+  const int W = (int)std::min<int64_t>(std::min(nr, 8), 46 * 1024 / std::max<int64_t>(per, 1));
+  if (W >= 1 && g.n_boxes > 0 && (nr + W - 1) / W <= 65535) {
+    k_rhs_box<<<dim3((unsigned)g.n_boxes, (unsigned)((nr + W - 1) / W)), 128, (size_t)(W * per), s>>>(g, khat, pol, nr,
+                                                                                                  W, rhs, ld);
+    return;
+  }
   int64_t blocks = ceil_div(total, 128);
   if (blocks > 152 * 64) blocks = 152 * 64;
-  k_rhs_pw<<<(unsigned)blocks, 128, 0, s>>>(V, T, area, tri_pm, free_pm, N, k, khat, pol, nr, rhs, ld);
+  k_rhs_pw<<<(unsigned)blocks, 128, 0, s>>>(g.V, g.T, g.area, g.tri_pm, g.free_pm, g.N, g.k, khat, pol, nr, rhs, ld);
 }
 
 // ---------------------------------------------------------------- Krylov

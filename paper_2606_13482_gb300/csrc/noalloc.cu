@@ -50,8 +50,7 @@ cudaError_t scratch_for_device(int dev, double** out) {
 
 namespace efie {
 // accessors implemented in api.cu (handle layout stays private there)
-int handle_rhs_args(const efie_handle* h, const double** V, const int32_t** T, const double** area,
-                    const int32_t** tri_pm, const int32_t** free_pm, int64_t* N, double* k, int* device);
+int handle_rhs_args(const efie_handle* h, RhsGeom* g, int* device);
 void handle_set_error(efie_handle* h, const char* msg);
 }  // namespace efie
 
@@ -68,12 +67,9 @@ extern "C" int efie_rhs_planewave_noalloc(efie_handle* h, int n_rhs, const doubl
     efie::handle_set_error(h, "efie_rhs_planewave_noalloc: NULL argument");
     return EFIE_EINVAL;
   }
-  const double *V, *area;
-  const int32_t *T, *tri_pm, *free_pm;
-  int64_t N;
-  double k;
+  efie::RhsGeom g;
   int hdev = 0, cur = -1;
-  if (efie::handle_rhs_args(h, &V, &T, &area, &tri_pm, &free_pm, &N, &k, &hdev) != EFIE_OK) return EFIE_EINVAL;
+  if (efie::handle_rhs_args(h, &g, &hdev) != EFIE_OK) return EFIE_EINVAL;
   if (cudaGetDevice(&cur) != cudaSuccess || cur != hdev) {
     efie::handle_set_error(h, ("efie_rhs_planewave_noalloc: the current device (" + std::to_string(cur) +
                                ") is not the handle's device (" + std::to_string(hdev) + ")").c_str());
@@ -92,8 +88,7 @@ extern "C" int efie_rhs_planewave_noalloc(efie_handle* h, int n_rhs, const doubl
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(scratch + 3 * kMaxPlaneWaves, pol, sizeof(double) * 3 * n_rhs, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) {
-    efie::launch_rhs_planewave(V, T, area, tri_pm, free_pm, N, k, scratch, scratch + 3 * kMaxPlaneWaves, n_rhs,
-                               (double2*)rhs, N, s);
+    efie::launch_rhs_planewave(g, scratch, scratch + 3 * kMaxPlaneWaves, n_rhs, (double2*)rhs, g.N, s);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // host inputs may be released after return
