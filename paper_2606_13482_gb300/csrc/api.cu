@@ -1573,7 +1573,7 @@ void setup_impl(efie_handle* h, const efie_mesh* mesh, double k, int p, double g
     const int64_t nblk = nd.n_blocks;
     const int64_t scr_cap = (int64_t)(1LL << 30) / (10 * 16);  // pairs per batch (~1 GiB)
     double2* scratch = nullptr;
-    int64_t* d_scr_off = M.alloc<int64_t>(nblk + 1);
+    int64_t* d_scr_off = M.alloc<int64_t>(nblk + 2);  // and the count of close pairs
     // T is symmetric: blocks (x, y) with x > y are copied as transposes of
     // (y, x) instead of being integrated.
     std::vector<int64_t> mir_blk, mir_src;
@@ -1613,7 +1613,12 @@ void setup_impl(efie_handle* h, const efie_mesh* mesh, double k, int p, double g
       }
       cuda_check(cudaMemcpy(d_scr_off, scr_off.data(), sizeof(int64_t) * scr_off.size(), cudaMemcpyHostToDevice),
                  "scr_off");
-      launch_near_pairs_A(nd, j0, j1 - j0, d_scr_off, scratch, scr_off.back(), s);
+      // the batch's list of close pairs lies in its A entries, which are formed
+      // afterwards: a box of n RWGs has at most 2 n triangles in its set, so a
+      // block has at most 4 pairs (4 bytes each) per entry (16 bytes)
+      launch_near_pairs_A(nd, j0, j1 - j0, d_scr_off, scratch, scr_off.back(),
+                          reinterpret_cast<uint32_t*>(nd.A + P.blkA_off[j0]),
+                          reinterpret_cast<uint32_t*>(d_scr_off + nblk + 1), s);
       launch_near_combine_A(nd, j0, j1 - j0, d_scr_off, scratch, P.blkA_off[j0],
                             P.blkA_off[j1] - P.blkA_off[j0], s);
       if (!h->direct)

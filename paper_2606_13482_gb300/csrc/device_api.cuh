@@ -42,8 +42,10 @@ struct NearDev {
 // transposes of the (y, x) blocks, copied by launch_near_mirror.
 
 int near_upload_rules(const double* q3, const double* q4);
+// close: room for total entries (the list of close pairs, *n_close of them); total below 2^32
 void launch_near_pairs_A(const NearDev& nd, int64_t j0, int64_t nblk, const int64_t* scr_off,
-                         double2* scratch, int64_t total, cudaStream_t s);
+                         double2* scratch, int64_t total, uint32_t* close, uint32_t* n_close,
+                         cudaStream_t s);
 void launch_near_combine_A(const NearDev& nd, int64_t j0, int64_t nblk, const int64_t* scr_off,
                            const double2* scratch, int64_t e_begin, int64_t total, cudaStream_t s);
 // V entries of the blocks j in [j0, j0 + nblk) (entries [e_begin, e_begin + total)),

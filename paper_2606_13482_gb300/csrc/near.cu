@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "device_api.cuh"
 
@@ -118,26 +120,50 @@ __device__ void static_pot(const TriG& g, const double* r, double& I1, double* I
     double vterm = 0.5 * (R0sq * lg + lp * Rp - lm * Rm);
     for (int d = 0; d < 3; ++d) Iv[d] += vterm * uh[d];
     if (fabs(P0) > 1e-300) {
-      double at = atan2(P0 * lp, R0sq + ad * Rp) - atan2(P0 * lm, R0sq + ad * Rm);
-      I1 += P0 * lg - ad * at;
+      // difference of two angles, each in (-pi/2, pi/2), as one
+      const double yp = P0 * lp, xp = R0sq + ad * Rp, ym = P0 * lm, xm = R0sq + ad * Rm;
+      I1 += P0 * lg - ad * atan2(yp * xm - ym * xp, xp * xm + yp * ym);
     }
   }
 }
 
-// (exp(-jkR) - 1)/(4 pi R), limit -jk/(4 pi) at R = 0
-__device__ __forceinline__ double2 smooth_rem(double R, double k) {
-  if (!(R > 0)) return make_double2(0.0, -k / FOUR_PI);
-  double s, c, sh, ch;
-  sincos(k * R, &s, &c);
-  sincos(0.5 * k * R, &sh, &ch);
-  return make_double2(-2.0 * sh * sh / (FOUR_PI * R), -s / (FOUR_PI * R));
+// Taylor series of cos(x) and sin(x) / x in q = x^2: below 1e-16 for |x| <= 1.25
+// (ten terms) or 0.65 (eight)
+template <int TERMS>
+__device__ __forceinline__ void cos_sinc_series(double q, double& cs, double& sc) {
+  double c, s;
+  if (TERMS == 10) {
+    c = -1.0 / 6402373705728000.0, s = -1.0 / 121645100408832000.0;  // 1/18!, 1/19!
+    c = fma(c, q, 1.0 / 20922789888000.0), s = fma(s, q, 1.0 / 355687428096000.0);
+    c = fma(c, q, -1.0 / 87178291200.0), s = fma(s, q, -1.0 / 1307674368000.0);
+  } else {
+    c = -1.0 / 87178291200.0, s = -1.0 / 1307674368000.0;  // 1/14!, 1/15!
+  }
+  c = fma(c, q, 1.0 / 479001600.0), s = fma(s, q, 1.0 / 6227020800.0);
+  c = fma(c, q, -1.0 / 3628800.0), s = fma(s, q, -1.0 / 39916800.0);
+  c = fma(c, q, 1.0 / 40320.0), s = fma(s, q, 1.0 / 362880.0);
+  c = fma(c, q, -1.0 / 720.0), s = fma(s, q, -1.0 / 5040.0);
+  c = fma(c, q, 1.0 / 24.0), s = fma(s, q, 1.0 / 120.0);
+  c = fma(c, q, -0.5), s = fma(s, q, -1.0 / 6.0);
+  cs = fma(c, q, 1.0);
+  sc = fma(s, q, 1.0);
 }
 
-__device__ __forceinline__ double2 green(double R, double k) {
-  double s, c;
-  sincos(k * R, &s, &c);
-  double f = 1.0 / (FOUR_PI * R);
-  return make_double2(c * f, -s * f);
+// (exp(-jkR) - 1)/(4 pi R) from R^2, limit -jk/(4 pi) at R = 0
+__device__ __forceinline__ double2 smooth_rem(double R2, double k) {
+  const double q = 0.25 * k * k * R2;
+  if (q <= 1.25 * 1.25) {
+    // with x = kR / 2, sin x = x P, cos x = Q: -2 sin^2 x / R = -k x P^2, -sin(kR) / R = -k P Q
+    double P, Q;
+    cos_sinc_series<10>(q, Q, P);
+    const double f = -k / FOUR_PI * P;
+    return make_double2(f * P * sqrt(q), f * Q);
+  }
+  const double R = sqrt(R2);
+  double sh, ch;
+  sincos(0.5 * k * R, &sh, &ch);
+  const double f = -2.0 * sh / (FOUR_PI * R);  // sin(kR) = 2 sin(kR/2) cos(kR/2)
+  return make_double2(f * sh, f * ch);
 }
 
 __device__ __forceinline__ bool is_close(const TriG& A, const TriG& B) {
@@ -173,7 +199,6 @@ __device__ void pair_close_oriented(const TriG& A, const TriG& B, double k, bool
         dd[d] = x[d] - ya[q][d];
         R += dd[d] * dd[d];
       }
-      R = sqrt(R);
       double2 s = smooth_rem(R, k);
       double wy = c_q4[2][q] * B.twoa;
       s.x *= wy;
@@ -208,7 +233,12 @@ __device__ void pair_close_oriented(const TriG& A, const TriG& B, double k, bool
   }
 }
 
-__device__ void pair_regular(const TriG& A, const TriG& B, double k, bool full, double2& I0,
+// The phase of a point pair is that of the centroids' distance Rc plus k (R - Rc),
+// which stays below k times the two triangles' extents: a series instead of a
+// full sine and cosine at each of the 81 point pairs, rotated by exp(-jk Rc) at the
+// end (elements above about lambda / 6 take the full functions).
+template <int TERMS>  // of the series; 0: full sine and cosine
+__device__ void pair_regular_t(const TriG& A, const TriG& B, double k, bool full, double2& I0,
                              double2* Ivv) {
   double ya[9][3], wy[9];
   for (int q = 0; q < 9; ++q) {
@@ -218,25 +248,35 @@ __device__ void pair_regular(const TriG& A, const TriG& B, double k, bool full, 
     wy[q] = c_q3[2][q] * B.twoa;
   }
   double dc[3] = {A.c[0] - B.c[0], A.c[1] - B.c[1], A.c[2] - B.c[2]};
+  const double Rc = sqrt(dc[0] * dc[0] + dc[1] * dc[1] + dc[2] * dc[2]);
   double2 J00 = make_double2(0, 0), Jx[3], Jy[3], Jxy = make_double2(0, 0);
   for (int d = 0; d < 3; ++d) Jx[d] = Jy[d] = make_double2(0, 0);
   for (int p = 0; p < 9; ++p) {
     double x[3], xl[3];
     rule_point(A, c_q3[0][p], c_q3[1][p], x);
-    for (int d = 0; d < 3; ++d) xl[d] = x[d] - A.c[d];
+    for (int d = 0; d < 3; ++d) {
+      xl[d] = x[d] - A.c[d];
+      x[d] = dc[d] + xl[d];
+    }
     double wx = c_q3[2][p] * A.twoa;
     double2 S = make_double2(0, 0), Sy[3];
     for (int d = 0; d < 3; ++d) Sy[d] = make_double2(0, 0);
     for (int q = 0; q < 9; ++q) {
       double R = 0;
       for (int d = 0; d < 3; ++d) {
-        double t = dc[d] + xl[d] - ya[q][d];
+        double t = x[d] - ya[q][d];
         R += t * t;
       }
-      R = sqrt(R);
-      double2 g = green(R, k);
-      g.x *= wy[q];
-      g.y *= wy[q];
+      const double ir = rsqrt(R);
+      const double f = ir * wy[q], ph = k * fma(R, ir, -Rc);
+      double sn, cs;
+      if constexpr (TERMS > 0) {
+        cos_sinc_series<TERMS>(ph * ph, cs, sn);
+        sn *= ph;
+      } else {
+        sincos(ph, &sn, &cs);
+      }
+      const double2 g = make_double2(cs * f, -sn * f);
       S.x += g.x;
       S.y += g.y;
       if (full)
@@ -257,6 +297,17 @@ __device__ void pair_regular(const TriG& A, const TriG& B, double k, bool full, 
         Jxy.y += wx * xl[d] * Sy[d].y;
       }
   }
+  {
+    double2 e;  // exp(-jk Rc) / (4 pi)
+    sincos(k * Rc, &e.y, &e.x);
+    e.x *= 1.0 / FOUR_PI;
+    e.y *= -1.0 / FOUR_PI;
+    J00 = cmul(J00, e);
+    if (full) {
+      for (int d = 0; d < 3; ++d) Jx[d] = cmul(Jx[d], e), Jy[d] = cmul(Jy[d], e);
+      Jxy = cmul(Jxy, e);
+    }
+  }
   I0 = J00;
   if (!full) return;
   for (int i = 0; i < 3; ++i)
@@ -276,6 +327,15 @@ __device__ void pair_regular(const TriG& A, const TriG& B, double k, bool full, 
       v.y += ab * J00.y;
       Ivv[3 * i + j] = v;
     }
+}
+
+__device__ __forceinline__ void pair_regular(const TriG& A, const TriG& B, double k, bool full, double2& I0,
+                                             double2* Ivv) {
+  // a triangle's points lie within its longest edge times 2 / 3 of its centroid
+  const double ext = k * (2.0 / 3.0) * (sqrt(A.emax2) + sqrt(B.emax2));
+  if (ext <= 0.65) pair_regular_t<8>(A, B, k, full, I0, Ivv);
+  else if (ext <= 1.25) pair_regular_t<10>(A, B, k, full, I0, Ivv);
+  else pair_regular_t<0>(A, B, k, full, I0, Ivv);
 }
 
 // Pair integrals of canonical triangles (ta, tb): I0 and (full) Ivv[9].
@@ -311,9 +371,16 @@ __device__ __forceinline__ int64_t find_block(const int64_t* off, int64_t n, int
 
 // ---------------------------------------------------------------- assembly
 // Triangle-pair integrals for the A blocks j in [j0, j1): pair (a, b) of the
-// triangle sets T_x x T_y; scratch[e] = {I0, Ivv[9]} (10 double2).
-__global__ void k_near_pairs_A(NearDev nd, int64_t j0, int64_t nblk, const int64_t* scr_off,
-                               double2* scratch, int64_t total) {
+// triangle sets T_x x T_y; scratch[e] = {I0, Ivv[9]} (10 double2).  Regular pairs
+// are integrated here; close ones (about 30 per triangle, each fifteen times a
+// regular one's work) go to a list, so that no warp waits for a few of them.
+//
+// What bounds it: the FP64 pipe (two operations per clock and SM).  With both
+// rules in one kernel and full sines and cosines the assembly of 12,000 unknowns
+// took 270 ms; now 47 for the regular pairs and 26 for the close ones.
+__global__ void __launch_bounds__(128) k_near_pairs_A(NearDev nd, int64_t j0, int64_t nblk, const int64_t* scr_off,
+                                                      double2* scratch, int64_t total, uint32_t* close,
+                                                      uint32_t* n_close) {
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   int64_t jl = find_block(scr_off, nblk, e);
@@ -322,13 +389,57 @@ __global__ void k_near_pairs_A(NearDev nd, int64_t j0, int64_t nblk, const int64
   int64_t ny = nd.tset_ptr[y + 1] - nd.tset_ptr[y];
   int64_t loc = e - scr_off[jl];
   int64_t a = loc / ny, b = loc - a * ny;
-  int ta = nd.tset[nd.tset_ptr[x] + a];
-  int tb = nd.tset[nd.tset_ptr[y] + b];
+  TriG A, B;
+  load_tri(nd.V, nd.T, nd.tset[nd.tset_ptr[x] + a], A);
+  load_tri(nd.V, nd.T, nd.tset[nd.tset_ptr[y] + b], B);
+  if (is_close(A, B)) {
+    close[atomicAdd(n_close, 1u)] = (uint32_t)e;  // the order does not matter: every pair has its own slot
+    return;
+  }
   double2 I0, Ivv[9];
-  pair_integrals(nd.V, nd.T, ta, tb, nd.k, true, I0, Ivv);
+  pair_regular(A, B, nd.k, true, I0, Ivv);
   double2* out = scratch + 10 * e;
   out[0] = I0;
   for (int q = 0; q < 9; ++q) out[1 + q] = Ivv[q];
+}
+
+// The listed close pairs: *n_close of them, two lanes per pair, one orientation each.
+__global__ void __launch_bounds__(128) k_near_pairs_close(NearDev nd, int64_t j0, int64_t nblk,
+                                                          const int64_t* scr_off, double2* scratch,
+                                                          const uint32_t* close, const uint32_t* n_close) {
+  const int64_t n = 2 * (int64_t)*n_close;
+  const int o = threadIdx.x & 1;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += stride) {
+    const int64_t i = i0 + threadIdx.x;
+    const bool ok = i < n;
+    const int64_t e = close[ok ? i >> 1 : 0];
+    int64_t jl = find_block(scr_off, nblk, e);
+    int64_t j = j0 + jl;
+    int32_t x = nd.blk_tgt[j], y = nd.near_src[j];
+    int64_t ny = nd.tset_ptr[y + 1] - nd.tset_ptr[y];
+    int64_t loc = e - scr_off[jl];
+    int64_t a = loc / ny, b = loc - a * ny;
+    const int ta = nd.tset[nd.tset_ptr[x] + a], tb = nd.tset[nd.tset_ptr[y] + b];
+    TriG A, B;
+    load_tri(nd.V, nd.T, o ? tb : ta, A);
+    load_tri(nd.V, nd.T, o ? ta : tb, B);
+    double2 I0, Ivv[9];
+    pair_close_oriented(A, B, nd.k, true, I0, Ivv);
+    // the mean of the two orientations, the second one transposed
+    double2* out = scratch + 10 * e;
+    const double2 J0 = make_double2(__shfl_xor_sync(0xffffffffu, I0.x, 1), __shfl_xor_sync(0xffffffffu, I0.y, 1));
+    if (ok && o == 0) out[0] = make_double2(0.5 * (I0.x + J0.x), 0.5 * (I0.y + J0.y));
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const double2 v = Ivv[3 * q + p];
+        const double2 t = make_double2(__shfl_xor_sync(0xffffffffu, v.x, 1), __shfl_xor_sync(0xffffffffu, v.y, 1));
+        if (ok && o == 0)
+          out[1 + 3 * p + q] = make_double2(0.5 * (Ivv[3 * p + q].x + t.x), 0.5 * (Ivv[3 * p + q].y + t.y));
+      }
+  }
 }
 
 // A block entries from the pair scratch:
@@ -358,9 +469,11 @@ __global__ void k_near_combine_A(NearDev nd, int64_t j0, int64_t nblk, const int
       double2 v = scr[10 * pe + 1 + 3 * nd.rwg_loc[2 * i + s] + nd.rwg_loc[2 * n + t]];
       acc.x += cf * v.x;
       acc.y += cf * v.y;
-      const double2 i0 = scr[10 * pe];
-      phi.x += 4.0 * cf * i0.x;
-      phi.y += 4.0 * cf * i0.y;
+      if (nd.Phi) {
+        const double2 i0 = scr[10 * pe];
+        phi.x += 4.0 * cf * i0.x;
+        phi.y += 4.0 * cf * i0.y;
+      }
     }
   nd.A[eg] = acc;
   if (nd.Phi) nd.Phi[eg] = phi;
@@ -922,9 +1035,13 @@ int near_upload_rules(const double* q3, const double* q4) {
 }
 
 void launch_near_pairs_A(const NearDev& nd, int64_t j0, int64_t nblk, const int64_t* scr_off,
-                         double2* scratch, int64_t total, cudaStream_t s) {
+                         double2* scratch, int64_t total, uint32_t* close, uint32_t* n_close, cudaStream_t s) {
   if (total <= 0) return;
-  k_near_pairs_A<<<(unsigned)ceil_div(total, 128), 128, 0, s>>>(nd, j0, nblk, scr_off, scratch, total);
+  cudaMemsetAsync(n_close, 0, sizeof(uint32_t), s);
+  k_near_pairs_A<<<(unsigned)ceil_div(total, 128), 128, 0, s>>>(nd, j0, nblk, scr_off, scratch, total, close,
+                                                               n_close);
+  k_near_pairs_close<<<(unsigned)std::min<int64_t>(ceil_div(2 * total, 128), 152 * 16), 128, 0, s>>>(
+      nd, j0, nblk, scr_off, scratch, close, n_close);
 }
 void launch_near_combine_A(const NearDev& nd, int64_t j0, int64_t nblk, const int64_t* scr_off,
                            const double2* scratch, int64_t e_begin, int64_t total, cudaStream_t s) {
