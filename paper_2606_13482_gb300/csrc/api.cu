@@ -128,6 +128,7 @@ struct FarSet {
     cpx_t<R>* Mf = nullptr;
     cpx_t<R>* Mb = nullptr;
     R *CL = nullptr, *CR = nullptr, *CLt = nullptr, *CRt = nullptr;
+    SparseMat<R> up, down;   // their nonzeros, where the fused transfers take them (nnz 0: dense passes)
     cpx_t<R>* Kh = nullptr;
     cpx_t<R>* KH[6] = {};  // dyadic factorization: Hessian spectra, ab = 00, 01, 02, 11, 12, 22
   };
@@ -180,6 +181,7 @@ struct LevDev {
           *ux_s1 = nullptr;
   int8_t *uz_b0 = nullptr, *uz_b1 = nullptr, *uy_b0 = nullptr, *uy_b1 = nullptr, *ux_b0 = nullptr,
          *ux_b1 = nullptr;
+  int32_t* child8 = nullptr;  // on a parent level: its children by half bits, [B][4 bx + 2 by + bz], -1: none
   int64_t *dx_src = nullptr, *dy_src = nullptr, *dz_src = nullptr;  // downward: g2 -> parent, g1 -> g2, child -> g1
   int8_t *dx_sel = nullptr, *dy_sel = nullptr;                      // [G][3]
   // leaves of the tree on this level (all boxes of level D in a uniform tree;
@@ -364,6 +366,10 @@ struct KScope {
       cudaEventRecord(a, s);
     }
   }
+  void launches(int n) {  // added to the count given at the start
+    h->n_launches += n;
+    if (h->prof.on) h->prof.launches[cls] += n;
+  }
   ~KScope() {
     if (a) {
       cudaEventRecord(b, s);
@@ -466,6 +472,25 @@ void build_far(efie_handle* h, FarSet<R>& F, cudaStream_t s) {
       FL.CR = M.upload(cr);
       FL.CLt = M.upload(clt);
       FL.CRt = M.upload(crt);
+      const auto sparse = [&](int rows, auto&& entry, int ncol) {  // entry(row, col) -> value
+        std::vector<int> ptr(1, 0), idx;
+        std::vector<R> coef;
+        for (int r = 0; r < rows; ++r) {
+          for (int c = 0; c < ncol; ++c) {
+            const R v = entry(r, c);
+            if (v != (R)0) idx.push_back(c), coef.push_back(v);
+          }
+          ptr.push_back((int)idx.size());
+        }
+        SparseMat<R> m;
+        const double per = (double)idx.size() / rows;
+        if (idx.empty() || per * per * per > TRANSFER_FUSED_LOADS<R> || idx.size() > 1024) return m;
+        m.rows = rows, m.nnz = (int)idx.size();
+        m.ptr = M.upload(ptr), m.idx = M.upload(idx), m.coef = M.upload(coef);
+        return m;
+      };
+      FL.up = sparse(spp, [&](int r, int c) { return (c & 1 ? cr : cl)[(size_t)r * sp + (c >> 1)]; }, 2 * sp);
+      FL.down = sparse(2 * sp, [&](int r, int c) { return (r < sp ? clt : crt)[(size_t)(r % sp) * spp + c]; }, spp);
     }
   }
   F.built = true;
@@ -729,23 +754,29 @@ void anterp_up(efie_handle* h, FarSet<R>& F, int nr, int rhs0, std::vector<cpx_t
   // y, x); a nonuniform tree's leaves on the parent level are anterpolated
   // after the transfer into that level, over its zeros
   for (int ell = D; ell > top; --ell) {
-    KScope ks(h, K_UP, s, 3);
+    KScope ks(h, K_UP, s, 0);
     const Level& L = P.L(ell);
     const Level& U = P.L(ell - 1);
     const LevDev& LD = h->lev[ell - top];
     auto& FL = F.lv[ell - top];
     const int64_t Bp = (int64_t)U.code.size();
     const int sp = L.sp, spp = U.sp;
-    View vq{(int64_t)sp * sp * sp * C, (int64_t)sp * sp * C, (int64_t)sp * C, C};
-    View t1{(int64_t)sp * sp * spp * C, (int64_t)sp * spp * C, (int64_t)spp * C, C};
-    View t2{(int64_t)sp * spp * spp * C, (int64_t)spp * spp * C, (int64_t)spp * C, C};
-    View vp{(int64_t)spp * spp * spp * C, (int64_t)spp * spp * C, (int64_t)spp * C, C};
-    launch_mode_pair<R>(qq[ell - top], vq, F.tmp1, t1, LD.ng1, C, 2, sp, sp, sp, spp, FL.CL, FL.CR, LD.uz_s0,
-                        LD.uz_s1, LD.uz_b0, LD.uz_b1, s);
-    launch_mode_pair<R>(F.tmp1, t1, F.tmp2, t2, LD.ng2, C, 1, sp, sp, spp, spp, FL.CL, FL.CR, LD.uy_s0,
-                        LD.uy_s1, LD.uy_b0, LD.uy_b1, s);
-    launch_mode_pair<R>(F.tmp2, t2, qq[ell - 1 - top], vp, Bp, C, 0, sp, spp, spp, spp, FL.CL, FL.CR, LD.ux_s0,
-                        LD.ux_s1, LD.ux_b0, LD.ux_b1, s);
+    if (FL.up.nnz) {
+      launch_up_fused<R>(qq[ell - top], qq[ell - 1 - top], Bp, C, sp, spp, FL.up, h->lev[ell - 1 - top].child8, s);
+      ks.launches(1);
+    } else {
+      View vq{(int64_t)sp * sp * sp * C, (int64_t)sp * sp * C, (int64_t)sp * C, C};
+      View t1{(int64_t)sp * sp * spp * C, (int64_t)sp * spp * C, (int64_t)spp * C, C};
+      View t2{(int64_t)sp * spp * spp * C, (int64_t)spp * spp * C, (int64_t)spp * C, C};
+      View vp{(int64_t)spp * spp * spp * C, (int64_t)spp * spp * C, (int64_t)spp * C, C};
+      launch_mode_pair<R>(qq[ell - top], vq, F.tmp1, t1, LD.ng1, C, 2, sp, sp, sp, spp, FL.CL, FL.CR, LD.uz_s0,
+                          LD.uz_s1, LD.uz_b0, LD.uz_b1, s);
+      launch_mode_pair<R>(F.tmp1, t1, F.tmp2, t2, LD.ng2, C, 1, sp, sp, spp, spp, FL.CL, FL.CR, LD.uy_s0,
+                          LD.uy_s1, LD.uy_b0, LD.uy_b1, s);
+      launch_mode_pair<R>(F.tmp2, t2, qq[ell - 1 - top], vp, Bp, C, 0, sp, spp, spp, spp, FL.CL, FL.CR, LD.ux_s0,
+                          LD.ux_s1, LD.ux_b0, LD.ux_b1, s);
+      ks.launches(3);
+    }
     anterp(ell - 1);
   }
 }
@@ -929,13 +960,19 @@ void down_interp(efie_handle* h, FarSet<R>& F, int nr, int rhs0, std::vector<cpx
   // downward transfers r_c += C^T r_parent (Sec. IV-B), shared among siblings one
   // axis at a time (x for (parent, b_x), y for (parent, b_x, b_y), z per child)
   for (int ell = top + 1; ell <= D; ++ell) {
-    KScope ks(h, K_DOWN, s, 3);
+    KScope ks(h, K_DOWN, s, 0);
     const Level& L = P.L(ell);
     const Level& U = P.L(ell - 1);
     const LevDev& LD = h->lev[ell - top];
     auto& FL = F.lv[ell - top];
     int64_t B = (int64_t)L.code.size();
     int sp = L.sp, spp = U.sp;
+    if (FL.down.nnz) {
+      launch_down_fused<R>(rr[ell - 1 - top], rr[ell - top], B, C, sp, spp, FL.down, LD.parent, LD.bits, s);
+      ks.launches(1);
+      continue;
+    }
+    ks.launches(3);
     View vp{(int64_t)spp * spp * spp * C, (int64_t)spp * spp * C, (int64_t)spp * C, C};
     View w1{(int64_t)sp * spp * spp * C, (int64_t)spp * spp * C, (int64_t)spp * C, C};
     View w2{(int64_t)sp * sp * spp * C, (int64_t)sp * spp * C, (int64_t)spp * C, C};
@@ -1390,7 +1427,15 @@ void setup_impl(efie_handle* h, const efie_mesh* mesh, double k, int p, double g
     for (int64_t b = 0; b < LD.B; ++b)
       for (int d = 0; d < 3; ++d) bits[3 * b + d] = (int8_t)(L.ijk[3 * b + d] & 1);
     LD.bits = M.upload(bits);
-    if (ell < P.D) LD.child_ptr = M.upload(L.child_ptr);
+    if (ell < P.D) {
+      LD.child_ptr = M.upload(L.child_ptr);
+      const Level& K = P.L(ell + 1);
+      std::vector<int32_t> c8(8 * LD.B, -1);
+      for (int64_t b = 0; b < LD.B; ++b)
+        for (int64_t c = L.child_ptr[b]; c < L.child_ptr[b + 1]; ++c)
+          c8[8 * b + 4 * (K.ijk[3 * c] & 1) + 2 * (K.ijk[3 * c + 1] & 1) + (K.ijk[3 * c + 2] & 1)] = (int32_t)c;
+      LD.child8 = M.upload(c8);
+    }
     if (ell > P.top) {
       const Level& U = P.L(ell - 1);
       const int64_t Bp = (int64_t)U.code.size();

@@ -119,6 +119,27 @@ void launch_mode_pair(const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, in
                       int e0, int e1, int e2, const R* M0, const R* M1, const int64_t* src0, const int64_t* src1,
                       const int8_t* bit0, const int8_t* bit1, cudaStream_t s);
 
+// Transfers by the nonzeros of their matrices, all three axes in one kernel.
+// Rows of the upward matrix [C^L C^R] (parent splines): entries 2 i + half over the
+// child splines i; rows of the downward one: half * sp + child spline, entries the
+// parent splines.  Entries ascend.
+template <typename R>
+struct SparseMat {
+  int rows = 0, nnz = 0;
+  const int* ptr = nullptr;
+  const int* idx = nullptr;
+  const R* coef = nullptr;
+};
+// loads per output point up to which the fused form is taken
+template <typename R>
+constexpr double TRANSFER_FUSED_LOADS = sizeof(R) == 4 ? 8 : 40;
+template <typename R>
+void launch_up_fused(const cpx_t<R>* q, cpx_t<R>* out, int64_t Bp, int C, int sp, int spp, const SparseMat<R>& m,
+                     const int32_t* child, cudaStream_t s);
+template <typename R>
+void launch_down_fused(const cpx_t<R>* r, cpx_t<R>* out, int64_t B, int C, int sp, int spp, const SparseMat<R>& m,
+                       const int64_t* parent, const int8_t* bits, cudaStream_t s);
+
 // DFT passes of the stabilized transforms using the conjugate symmetry of
 // M = F P (forward, n x nin) / P^T F^{-1} (inverse, nout x n); false when no
 // specialisation fits

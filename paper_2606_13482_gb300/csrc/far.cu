@@ -572,6 +572,193 @@ void launch_mode_pair(const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, in
   throw EfieError{EFIE_EINVAL, "transfer: more than 40 splines per axis below the top level"};
 }
 
+// ---------------------------------------------------------------- fused sparse transfers
+// Knot insertion touches few splines: where s doubles, a transfer matrix has
+// little more than one nonzero per child spline (12 of 117 for 9 -> 13 splines).
+// A thread owns 16 bytes (two FP32 channels or one FP64) of an output point and
+// takes the nested sums over the nonzeros of its three matrix rows straight from
+// the source grids, so the intermediates of the axis-by-axis passes never exist.
+// The sums run in the passes' order (z inside y inside x; both children of an
+// index before the next index) and leave out exact zeros only, so the results
+// are theirs bit for bit.
+//
+// What bounds it: the chains of dependent loads, (nonzeros per row)^3 of 16 bytes
+// per output -- 6.3 upward and 2.4 downward on average for 9 -> 13 splines, up to 216
+// at a parent's centre.  So in FP32 rows of more than 8 loads keep the passes (11 -> 15
+// splines, 22 upward: 0.31 ms in passes, 0.76 fused; 7 downward: 0.33 and 0.31); in
+// FP64, where the passes multiply every zero on a pipe of two operations per
+// clock, up to 40.  Dense constant-s transfers (three nonzeros per child spline)
+// keep the passes.  Measured, ms, upward and downward: 10-wavelength sphere, FP32,
+// 64 vectors 10.2 -> 8.2 and 10.2 -> 6.3; 4-wavelength sphere, FP64, 8 vectors 1.67 ->
+// 0.28 and 1.29 -> 0.23.
+template <typename R>
+struct U16;
+template <>
+struct U16<float> {
+  using T = float4;
+  static __device__ __forceinline__ T zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+  static __device__ __forceinline__ void fma1(float c, const T& v, T& a) {
+    a.x = fmaf(c, v.x, a.x), a.y = fmaf(c, v.y, a.y), a.z = fmaf(c, v.z, a.z), a.w = fmaf(c, v.w, a.w);
+  }
+  static __device__ __forceinline__ T add(const T& a, const T& b) {
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+  }
+};
+template <>
+struct U16<double> {
+  using T = double2;
+  static __device__ __forceinline__ T zero() { return make_double2(0.0, 0.0); }
+  static __device__ __forceinline__ void fma1(double c, const T& v, T& a) {
+    a.x = fma(c, v.x, a.x), a.y = fma(c, v.y, a.y);
+  }
+  static __device__ __forceinline__ T add(const T& a, const T& b) { return make_double2(a.x + b.x, a.y + b.y); }
+};
+
+// ptr [rows + 1], then idx and coef of the entries, into shared memory
+template <typename R>
+struct SparseRows {
+  const int* ptr;
+  const int* idx;
+  const R* coef;
+};
+template <typename R>
+__device__ __forceinline__ SparseRows<R> stage_rows(const SparseMat<R>& m, unsigned char* smem) {
+  R* coef = reinterpret_cast<R*>(smem);
+  int* idx = reinterpret_cast<int*>(coef + m.nnz);
+  int* ptr = idx + m.nnz;
+  for (int i = threadIdx.x; i < m.nnz; i += blockDim.x) coef[i] = m.coef[i], idx[i] = m.idx[i];
+  for (int i = threadIdx.x; i <= m.rows; i += blockDim.x) ptr[i] = m.ptr[i];
+  __syncthreads();
+  return {ptr, idx, coef};
+}
+
+// parent grids from their children (child[8 pb + 4 bx + 2 by + bz], -1: none);
+// entries of a row: child index * 2 + half, ascending
+template <typename R>
+__global__ void __launch_bounds__(256) k_up_fused(const typename U16<R>::T* __restrict__ q,
+                                                  typename U16<R>::T* __restrict__ out, int ppb, int nb, int U, int sp,
+                                                  int spp, const SparseMat<R> m, const int32_t* __restrict__ child) {
+  using T = typename U16<R>::T;
+  extern __shared__ __align__(16) unsigned char up_smem[];
+  const SparseRows<R> rows = stage_rows(m, up_smem);
+  const int64_t pb = blockIdx.x / nb;
+  const int p0 = (int)(blockIdx.x - pb * nb) * ppb, npt = spp * spp * spp, csz = sp * sp * sp * U;
+  int ch[8];
+  {
+    const int4 c0 = __ldg(reinterpret_cast<const int4*>(child + 8 * pb)),
+               c1 = __ldg(reinterpret_cast<const int4*>(child + 8 * pb) + 1);
+    ch[0] = c0.x, ch[1] = c0.y, ch[2] = c0.z, ch[3] = c0.w, ch[4] = c1.x, ch[5] = c1.y, ch[6] = c1.z, ch[7] = c1.w;
+  }
+  for (int e = threadIdx.x; e < ppb * U; e += blockDim.x) {
+    const int pt = p0 + e / U, u = e % U;
+    if (pt >= npt) break;
+    const int Z = pt % spp, Y = (pt / spp) % spp, X = pt / (spp * spp);
+    const int z0 = rows.ptr[Z], z1 = rows.ptr[Z + 1];
+    T ax = U16<R>::zero();
+    for (int ex = rows.ptr[X]; ex < rows.ptr[X + 1]; ++ex) {
+      const int i = rows.idx[ex] >> 1;
+      const bool bx = rows.idx[ex] & 1;
+      const int h0 = bx ? ch[4] : ch[0], h1 = bx ? ch[5] : ch[1], h2 = bx ? ch[6] : ch[2], h3 = bx ? ch[7] : ch[3];
+      if ((h0 & h1 & h2 & h3) < 0) continue;  // no child on this side (-1 each)
+      T ay = U16<R>::zero();
+      for (int ey = rows.ptr[Y]; ey < rows.ptr[Y + 1]; ++ey) {
+        const int j = rows.idx[ey] >> 1;
+        const bool by = rows.idx[ey] & 1;
+        const int g0 = by ? h2 : h0, g1 = by ? h3 : h1;
+        if ((g0 & g1) < 0) continue;
+        // an absent child's terms are exact zeros: its sibling's values, coefficient 0
+        const T* q0 = q + (int64_t)(g0 < 0 ? g1 : g0) * csz + (i * sp + j) * sp * U + u;
+        const T* q1 = q + (int64_t)(g1 < 0 ? g0 : g1) * csz + (i * sp + j) * sp * U + u;
+        T az = U16<R>::zero();
+#pragma unroll 3
+        for (int ez = z0; ez < z1; ++ez) {
+          const int k = rows.idx[ez] >> 1;
+          const bool bz = rows.idx[ez] & 1;
+          const R c = (bz ? g1 : g0) < 0 ? (R)0 : rows.coef[ez];
+          U16<R>::fma1(c, __ldg((bz ? q1 : q0) + k * U), az);
+        }
+        U16<R>::fma1(rows.coef[ey], az, ay);
+      }
+      U16<R>::fma1(rows.coef[ex], ay, ax);
+    }
+    out[(pb * npt + pt) * U + u] = ax;
+  }
+}
+
+// child grids += their parents' (rows of m: half * sp + child spline, entries the
+// parent splines ascending)
+template <typename R>
+__global__ void __launch_bounds__(256) k_down_fused(const typename U16<R>::T* __restrict__ r,
+                                                    typename U16<R>::T* __restrict__ out, int ppb, int nb, int U,
+                                                    int sp, int spp, const SparseMat<R> m,
+                                                    const int64_t* __restrict__ parent,
+                                                    const int8_t* __restrict__ bits) {
+  using T = typename U16<R>::T;
+  extern __shared__ __align__(16) unsigned char down_smem[];
+  const SparseRows<R> rows = stage_rows(m, down_smem);
+  const int64_t b = blockIdx.x / nb;
+  const int p0 = (int)(blockIdx.x - b * nb) * ppb, npt = sp * sp * sp;
+  const int kz = bits[3 * b + 2] ? sp : 0, ky = bits[3 * b + 1] ? sp : 0, kx = bits[3 * b] ? sp : 0;
+  const T* rb = r + parent[b] * ((int64_t)spp * spp * spp * U);
+  for (int e = threadIdx.x; e < ppb * U; e += blockDim.x) {
+    const int pt = p0 + e / U, u = e % U;
+    if (pt >= npt) break;
+    const int k = pt % sp + kz, j = (pt / sp) % sp + ky, i = pt / (sp * sp) + kx;
+    const int x0 = rows.ptr[i], x1 = rows.ptr[i + 1];
+    T* op = out + (b * npt + pt) * U + u;
+    const T old = *op;
+    T az = U16<R>::zero();
+    for (int ez = rows.ptr[k]; ez < rows.ptr[k + 1]; ++ez) {
+      const int Z = rows.idx[ez];
+      T ay = U16<R>::zero();
+      for (int ey = rows.ptr[j]; ey < rows.ptr[j + 1]; ++ey) {
+        const T* rp = rb + (rows.idx[ey] * spp + Z) * U + u;
+        T ax = U16<R>::zero();
+#pragma unroll 3
+        for (int ex = x0; ex < x1; ++ex)
+          U16<R>::fma1(rows.coef[ex], __ldg(rp + rows.idx[ex] * (spp * spp * U)), ax);
+        U16<R>::fma1(rows.coef[ey], ax, ay);
+      }
+      U16<R>::fma1(rows.coef[ez], ay, az);
+    }
+    *op = U16<R>::add(az, old);
+  }
+}
+
+template <typename R>
+static size_t rows_smem(const SparseMat<R>& m) {
+  return (size_t)m.nnz * (sizeof(R) + sizeof(int)) + sizeof(int) * (size_t)(m.rows + 1);
+}
+template <typename R>
+void launch_up_fused(const cpx_t<R>* q, cpx_t<R>* out, int64_t Bp, int C, int sp, int spp, const SparseMat<R>& m,
+                     const int32_t* child, cudaStream_t s) {
+  using T = typename U16<R>::T;
+  const int U = C * (int)sizeof(cpx_t<R>) / 16;
+  if (Bp <= 0) return;
+  // blocks of 1,024 units of one parent box (fewer where the boxes alone leave the chip empty)
+  const int npt = spp * spp * spp;
+  int ppb = std::max(1, 1024 / U);
+  while (ppb > 1 && ppb * U > 256 && Bp * ceil_div(npt, ppb) < 152 * 8) ppb /= 2;
+  const int nb = (int)ceil_div(npt, ppb);
+  k_up_fused<R><<<(unsigned)(Bp * nb), 256, rows_smem(m), s>>>(reinterpret_cast<const T*>(q),
+                                                               reinterpret_cast<T*>(out), ppb, nb, U, sp, spp, m,
+                                                               child);
+}
+template <typename R>
+void launch_down_fused(const cpx_t<R>* r, cpx_t<R>* out, int64_t B, int C, int sp, int spp, const SparseMat<R>& m,
+                       const int64_t* parent, const int8_t* bits, cudaStream_t s) {
+  using T = typename U16<R>::T;
+  const int U = C * (int)sizeof(cpx_t<R>) / 16;
+  if (B <= 0) return;
+  const int npt = sp * sp * sp;
+  int ppb = std::max(1, 1024 / U);
+  while (ppb > 1 && ppb * U > 256 && B * ceil_div(npt, ppb) < 152 * 8) ppb /= 2;
+  const int nb = (int)ceil_div(npt, ppb);
+  k_down_fused<R><<<(unsigned)(B * nb), 256, rows_smem(m), s>>>(reinterpret_cast<const T*>(r),
+                                                                reinterpret_cast<T*>(out), ppb, nb, U, sp, spp, m,
+                                                                parent, bits);
+}
+
 // ---------------------------------------------------------------- DFT passes
 // The transform passes apply M = F P (forward, n x s') or M = P^T F^{-1}
 // (inverse, s' x n) along one axis, F the n-point DFT and P real.  Because F's
@@ -2418,6 +2605,14 @@ void launch_norms(const double2* w, int64_t ldw, int64_t N, int nr, double* out,
 }
 
 // explicit instantiations
+template void launch_up_fused<float>(const float2*, float2*, int64_t, int, int, int, const SparseMat<float>&,
+                                     const int32_t*, cudaStream_t);
+template void launch_up_fused<double>(const double2*, double2*, int64_t, int, int, int, const SparseMat<double>&,
+                                      const int32_t*, cudaStream_t);
+template void launch_down_fused<float>(const float2*, float2*, int64_t, int, int, int, const SparseMat<float>&,
+                                       const int64_t*, const int8_t*, cudaStream_t);
+template void launch_down_fused<double>(const double2*, double2*, int64_t, int, int, int, const SparseMat<double>&,
+                                        const int64_t*, const int8_t*, cudaStream_t);
 template void launch_mode_pair<float>(const float2*, View, float2*, View, int64_t, int, int, int, int, int, int,
                                       const float*, const float*, const int64_t*, const int64_t*, const int8_t*,
                                       const int8_t*, cudaStream_t);
