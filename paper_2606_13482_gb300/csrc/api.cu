@@ -127,6 +127,7 @@ struct FarSet {
   struct Lev {
     cpx_t<R>* Mf = nullptr;
     cpx_t<R>* Mb = nullptr;
+    bool folded = false;     // FP64: Mf and Mb turned by the phases of launch_dft_fold
     R *CL = nullptr, *CR = nullptr, *CLt = nullptr, *CRt = nullptr;
     SparseMat<R> up, down;   // their nonzeros, where the fused transfers take them (nnz 0: dense passes)
     cpx_t<R>* Kh = nullptr;
@@ -456,6 +457,39 @@ void build_far(efie_handle* h, FarSet<R>& F, cudaStream_t s) {
     std::vector<cpx_t<R>> mf(L.Mf.size()), mb(L.Mb.size());
     for (size_t i = 0; i < mf.size(); ++i) mf[i] = mk<R>((R)L.Mf[i].real(), (R)L.Mf[i].imag());
     for (size_t i = 0; i < mb.size(); ++i) mb[i] = mk<R>((R)L.Mb[i].real(), (R)L.Mb[i].imag());
+    if constexpr (sizeof(R) == 8) {
+      // turned by theta_f = -pi f (shat - 1) / n, theta_{n-f} = -theta_f, where the mirror
+      // symmetry holds (P symmetric to rounding, n odd)
+      const int n = L.nfft, sp = L.sp;
+      std::vector<cplx> hf(L.Mf), hb(L.Mb);
+      double off = 0, big = 0;
+      for (int f = 0; f < n; ++f) {
+        const int g = 2 * f < n ? f : n - f;
+        double th = -3.14159265358979323846 * (double)(((int64_t)g * (L.shat - 1)) % (2 * n)) / n;
+        if (g != f) th = -th;
+        for (int j = 0; j < sp; ++j) {
+          hf[(size_t)f * sp + j] *= std::polar(1.0, -th);
+          hb[(size_t)j * n + f] *= std::polar(1.0, th);
+        }
+        for (int j = 0; j < sp; ++j) {
+          off = std::max({off, std::abs(hf[(size_t)f * sp + j] - std::conj(hf[(size_t)f * sp + sp - 1 - j])),
+                          n * std::abs(hb[(size_t)j * n + f] - std::conj(hb[(size_t)(sp - 1 - j) * n + f]))});
+          big = std::max(big, std::abs(hf[(size_t)f * sp + j]));
+        }
+      }
+      FL.folded = n % 2 == 1 && off <= 1e-13 * big;
+      if (FL.folded) {
+        // the folded passes read one half: make both halves exactly conjugate
+        for (int f = 0; f < n; ++f)
+          for (int j = 0; j < sp; ++j) {
+            const int q = sp - 1 - j;
+            const cplx a = 0.5 * (hf[(size_t)f * sp + j] + std::conj(hf[(size_t)f * sp + q]));
+            const cplx b = 0.5 * (hb[(size_t)j * n + f] + std::conj(hb[(size_t)q * n + f]));
+            mf[(size_t)f * sp + j] = make_double2(a.real(), a.imag());
+            mb[(size_t)j * n + f] = make_double2(b.real(), b.imag());
+          }
+      }
+    }
     FL.Mf = M.upload(mf);
     FL.Mb = M.upload(mb);
     if (ell > P.top) {
@@ -797,16 +831,27 @@ void fwd_level(efie_handle* h, FarSet<R>& F, int ell, int C, const cpx_t<R>* qin
                     (h->fft_variant == 1 || h->fft_variant == 2 || (h->fft_variant == 3 && sp == 9)) &&
                     dft_yz_fits(sp, n);
   KScope ks(h, K_FWD, s, fuse ? 2 : 3);
-  if (!launch_dft<R>(qin, vq, F.tmp1, a1, B, C, 0, sp, n, sp, sp, FL.Mf, n, false, s))
+  if (!dft_pass<R>(FL, qin, vq, F.tmp1, a1, B, C, 0, sp, n, sp, sp, n, false, s))
     launch_mode<R>(qin, vq, F.tmp1, a1, B, C, 0, sp, n, sp, sp, FL.Mf, FL.Mf, true, nullptr, nullptr, false, s);
   if (fuse &&
       launch_dft_yz(reinterpret_cast<const float2*>(F.tmp1), reinterpret_cast<float2*>(Qout), B, sp, n,
                     reinterpret_cast<const float2*>(FL.Mf), false, s))
     return;
-  if (!launch_dft<R>(F.tmp1, a1, F.tmp2, a2, B, C, 1, sp, n, n, sp, FL.Mf, n, false, s))
+  if (!dft_pass<R>(FL, F.tmp1, a1, F.tmp2, a2, B, C, 1, sp, n, n, sp, n, false, s))
     launch_mode<R>(F.tmp1, a1, F.tmp2, a2, B, C, 1, sp, n, n, sp, FL.Mf, FL.Mf, true, nullptr, nullptr, false, s);
-  if (!launch_dft<R>(F.tmp2, a2, Qout, vf, B, C, 2, sp, n, n, n, FL.Mf, n, false, s))
+  if (!dft_pass<R>(FL, F.tmp2, a2, Qout, vf, B, C, 2, sp, n, n, n, n, false, s))
     launch_mode<R>(F.tmp2, a2, Qout, vf, B, C, 2, sp, n, n, n, FL.Mf, FL.Mf, true, nullptr, nullptr, false, s);
+}
+
+// one transform pass: folded (FP64), or with the conjugate pairing; false when
+// neither takes it
+template <typename R, typename FL_>
+bool dft_pass(const FL_& FL, const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, int64_t B, int C, int ax, int nin,
+              int e0, int e1, int e2, int n, bool inverse, cudaStream_t s) {
+  const cpx_t<R>* M = inverse ? FL.Mb : FL.Mf;
+  if constexpr (sizeof(R) == 8)
+    if (FL.folded && launch_dft_fold(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n, inverse, s)) return true;
+  return launch_dft<R>(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n, inverse, s);
 }
 
 template <typename R>
@@ -828,15 +873,15 @@ void inv_level(efie_handle* h, FarSet<R>& F, int ell, int C, const cpx_t<R>* Rin
       launch_dft_yz(reinterpret_cast<const float2*>(Rin), reinterpret_cast<float2*>(F.tmp1), B, sp, n,
                     reinterpret_cast<const float2*>(FL.Mb), true, s)) {
     View vt{(int64_t)n * sp * sp * C, (int64_t)sp * sp * C, (int64_t)sp * C, C};
-    if (!launch_dft<R>(F.tmp1, vt, rout, vq, B, C, 0, n, sp, sp, sp, FL.Mb, n, true, s))
+    if (!dft_pass<R>(FL, F.tmp1, vt, rout, vq, B, C, 0, n, sp, sp, sp, n, true, s))
       launch_mode<R>(F.tmp1, vt, rout, vq, B, C, 0, n, sp, sp, sp, FL.Mb, FL.Mb, true, nullptr, nullptr, false, s);
     return;
   }
-  if (!launch_dft<R>(Rin, vf, F.tmp1, b1, B, C, 0, n, sp, n, n, FL.Mb, n, true, s))
+  if (!dft_pass<R>(FL, Rin, vf, F.tmp1, b1, B, C, 0, n, sp, n, n, n, true, s))
     launch_mode<R>(Rin, vf, F.tmp1, b1, B, C, 0, n, sp, n, n, FL.Mb, FL.Mb, true, nullptr, nullptr, false, s);
-  if (!launch_dft<R>(F.tmp1, b1, F.tmp2, b2, B, C, 1, n, sp, sp, n, FL.Mb, n, true, s))
+  if (!dft_pass<R>(FL, F.tmp1, b1, F.tmp2, b2, B, C, 1, n, sp, sp, n, n, true, s))
     launch_mode<R>(F.tmp1, b1, F.tmp2, b2, B, C, 1, n, sp, sp, n, FL.Mb, FL.Mb, true, nullptr, nullptr, false, s);
-  if (!launch_dft<R>(F.tmp2, b2, rout, vq, B, C, 2, n, sp, sp, sp, FL.Mb, n, true, s))
+  if (!dft_pass<R>(FL, F.tmp2, b2, rout, vq, B, C, 2, n, sp, sp, sp, n, true, s))
     launch_mode<R>(F.tmp2, b2, rout, vq, B, C, 2, n, sp, sp, sp, FL.Mb, FL.Mb, true, nullptr, nullptr, false, s);
 }
 

@@ -146,6 +146,9 @@ void launch_down_fused(const cpx_t<R>* r, cpx_t<R>* out, int64_t B, int C, int s
 template <typename R>
 bool launch_dft(const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, int64_t B, int C, int ax, int nin,
                 int e0, int e1, int e2, const cpx_t<R>* M, int n, bool inverse, cudaStream_t s);
+// the FP64 pass with the mirror symmetry of turned matrices as well
+bool launch_dft_fold(const double2* in, View vin, double2* out, View vout, int64_t B, int C, int ax, int nin, int e0,
+                     int e1, int e2, const double2* M, int n, bool inverse, cudaStream_t s);
 // fused second and third transform passes, FP32, 32 channels, on (box,
 // x-frequency) slabs; false when they do not apply
 bool launch_dft_yz(const float2* in, float2* out, int64_t B, int sp, int n, const float2* M, bool inverse,

@@ -935,6 +935,170 @@ __global__ void k_dft_inv_line(const cpx_t<R>* __restrict__ in, View vin, cpx_t<
   }
 }
 
+// FP64 passes with the mirror symmetry as well.  P is symmetric under reversal of
+// both its axes, so with the rows of M turned by a phase, H[f] = e^{-i theta_f} M[f],
+// e^{2 i theta_f} = w^{f (shat - 1)}, H[f][s' - 1 - j] = conj(H[f][j]): inputs j and s' - 1 - j
+// fold into u = v_j + v_j', w = v_j - v_j' and
+//   y_f = P1 + i P2, y_{n-f} = P1 - i P2,  P1 = sum Re H u, P2 = sum Im H w,
+// half the multiply-adds of the conjugate pairing alone; the outputs of the inverse
+// pass fold the same way.  The phases of the forward and the inverse pass
+// cancel across the translation, which multiplies frequency by frequency, so
+// spectra are simply kept turned.  FP64 is bound by its pipe (two operations per
+// clock and SM).  4-wavelength sphere, 8 vectors, ms: forward 6.0 -> 3.6, inverse
+// 5.9 -> 3.4.  (FP32 passes are bound by memory and keep their order of sums.)
+// Blocks of one warp where larger ones would leave SMs without work.
+template <int NH>
+__global__ void __launch_bounds__(128) k_dft_fwd_fold(const double2* __restrict__ in, View vin,
+                                                      double2* __restrict__ out, View vout, int64_t B, int C, int ax,
+                                                      int nin, int e0, int e1, int e2, const double2* __restrict__ M,
+                                                      int n) {
+  extern __shared__ unsigned char smem_raw[];
+  double2* Ms = reinterpret_cast<double2*>(smem_raw);  // [f][h], f = 0 .. n/2, h = columns 0 .. (nin - 1) / 2
+  const int nh = n / 2 + 1, hc = (nin + 1) / 2, half = nin / 2;
+  for (int i = threadIdx.x; i < nh * hc; i += blockDim.x) Ms[i] = M[(i / hc) * nin + i % hc];
+  __syncthreads();
+  const int ea = ax == 0 ? e1 : e0, eb = ax == 2 ? e1 : e2;
+  const int64_t sa_in = ax == 0 ? vin.s1 : vin.s0, sb_in = ax == 2 ? vin.s1 : vin.s2;
+  const int64_t sa_out = ax == 0 ? vout.s1 : vout.s0, sb_out = ax == 2 ? vout.s1 : vout.s2;
+  const int64_t step_in = ax == 0 ? vin.s0 : (ax == 1 ? vin.s1 : vin.s2);
+  const int64_t step_out = ax == 0 ? vout.s0 : (ax == 1 ? vout.s1 : vout.s2);
+  const int64_t lines = B * ea * eb * (int64_t)C;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < lines;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    int64_t t = idx;
+    const int c = (int)(t % C);
+    t /= C;
+    const int ib = (int)(t % eb);
+    t /= eb;
+    const int ia = (int)(t % ea);
+    const int64_t b = t / ea;
+    const double2* ip = in + b * vin.sb + ia * sa_in + ib * sb_in + c;
+    double2 u[NH], w[NH], mid = make_double2(0, 0);
+#pragma unroll
+    for (int j = 0; j < NH; ++j)
+      if (j < half) {
+        const double2 p = ip[j * step_in], q = ip[(int64_t)(nin - 1 - j) * step_in];
+        u[j] = cadd(p, q);
+        w[j] = csub(p, q);
+      }
+    if (hc > half) mid = ip[half * step_in];
+    double2* op = out + b * vout.sb + ia * sa_out + ib * sb_out + c;
+    for (int f = 0; f < nh; ++f) {
+      const double2* Mr = Ms + f * hc;
+      double2 p1 = make_double2(0, 0), p2 = p1;
+#pragma unroll
+      for (int j = 0; j < NH; ++j)
+        if (j < half) {
+          const double2 m = Mr[j];
+          p1.x = fma(m.x, u[j].x, p1.x);
+          p1.y = fma(m.x, u[j].y, p1.y);
+          p2.x = fma(m.y, w[j].x, p2.x);
+          p2.y = fma(m.y, w[j].y, p2.y);
+        }
+      if (hc > half) {
+        const double m = Mr[half].x;
+        p1.x = fma(m, mid.x, p1.x);
+        p1.y = fma(m, mid.y, p1.y);
+      }
+      op[f * step_out] = make_double2(p1.x - p2.y, p1.y + p2.x);
+      if (f != 0) op[(int64_t)(n - f) * step_out] = make_double2(p1.x + p2.y, p1.y - p2.x);
+    }
+  }
+}
+template <int NH>
+__global__ void __launch_bounds__(128) k_dft_inv_fold(const double2* __restrict__ in, View vin,
+                                                      double2* __restrict__ out, View vout, int64_t B, int C, int ax,
+                                                      int e0, int e1, int e2, const double2* __restrict__ M, int n) {
+  extern __shared__ unsigned char smem_raw[];
+  double2* Ms = reinterpret_cast<double2*>(smem_raw);  // [f][a], f = 0 .. n/2, a = 0 .. (nout - 1) / 2
+  const int nout = ax == 0 ? e0 : (ax == 1 ? e1 : e2);
+  const int nh = n / 2 + 1, hc = (nout + 1) / 2, half = nout / 2;
+  for (int i = threadIdx.x; i < nh * hc; i += blockDim.x) Ms[i] = M[(int64_t)(i % hc) * n + i / hc];
+  __syncthreads();
+  const int ea = ax == 0 ? e1 : e0, eb = ax == 2 ? e1 : e2;
+  const int64_t sa_in = ax == 0 ? vin.s1 : vin.s0, sb_in = ax == 2 ? vin.s1 : vin.s2;
+  const int64_t sa_out = ax == 0 ? vout.s1 : vout.s0, sb_out = ax == 2 ? vout.s1 : vout.s2;
+  const int64_t step_in = ax == 0 ? vin.s0 : (ax == 1 ? vin.s1 : vin.s2);
+  const int64_t step_out = ax == 0 ? vout.s0 : (ax == 1 ? vout.s1 : vout.s2);
+  const int64_t lines = B * ea * eb * (int64_t)C;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < lines;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    int64_t t = idx;
+    const int c = (int)(t % C);
+    t /= C;
+    const int ib = (int)(t % eb);
+    t /= eb;
+    const int ia = (int)(t % ea);
+    const int64_t b = t / ea;
+    const double2* ip = in + b * vin.sb + ia * sa_in + ib * sb_in + c;
+    double2 E[NH], O[NH], mid = make_double2(0, 0);
+    const double2 v0 = ip[0];
+#pragma unroll
+    for (int a = 0; a < NH; ++a)
+      if (a < half) {
+        E[a] = make_double2(Ms[a].x * v0.x, Ms[a].x * v0.y);
+        O[a] = make_double2(0, 0);
+      }
+    if (hc > half) mid = make_double2(Ms[half].x * v0.x, Ms[half].x * v0.y);
+    double2 z1 = nh > 1 ? ip[step_in] : v0, z2 = nh > 1 ? ip[(int64_t)(n - 1) * step_in] : v0;
+    for (int f = 1; f < nh; ++f) {
+      const double2 u = cadd(z1, z2), w = csub(z1, z2);
+      if (f + 1 < nh) {  // next pair's loads in flight during this pair's products
+        z1 = ip[(int64_t)(f + 1) * step_in];
+        z2 = ip[(int64_t)(n - f - 1) * step_in];
+      }
+      const double2* Mr = Ms + f * hc;
+#pragma unroll
+      for (int a = 0; a < NH; ++a)
+        if (a < half) {
+          const double2 m = Mr[a];
+          E[a].x = fma(m.x, u.x, E[a].x);
+          E[a].y = fma(m.x, u.y, E[a].y);
+          O[a].x = fma(m.y, w.x, O[a].x);
+          O[a].y = fma(m.y, w.y, O[a].y);
+        }
+      if (hc > half) {
+        mid.x = fma(Mr[half].x, u.x, mid.x);
+        mid.y = fma(Mr[half].x, u.y, mid.y);
+      }
+    }
+    double2* op = out + b * vout.sb + ia * sa_out + ib * sb_out + c;
+#pragma unroll
+    for (int a = 0; a < NH; ++a)
+      if (a < half) {
+        op[a * step_out] = make_double2(E[a].x - O[a].y, E[a].y + O[a].x);
+        op[(int64_t)(nout - 1 - a) * step_out] = make_double2(E[a].x + O[a].y, E[a].y - O[a].x);
+      }
+    if (hc > half) op[half * step_out] = mid;
+  }
+}
+
+// the folded pass, for turned matrices (see above) of odd length n and up to 21
+// splines; false where it does not apply
+bool launch_dft_fold(const double2* in, View vin, double2* out, View vout, int64_t B, int C, int ax, int nin, int e0,
+                     int e1, int e2, const double2* M, int n, bool inverse, cudaStream_t s) {
+  const int ea = ax == 0 ? e1 : e0, eb = ax == 2 ? e1 : e2;
+  const int ns = inverse ? (ax == 0 ? e0 : (ax == 1 ? e1 : e2)) : nin, half = ns / 2;
+  const int64_t lines = B * ea * eb * (int64_t)C;
+  if (half > 10 || n % 2 == 0) return false;
+  if (lines <= 0) return true;
+  const size_t smem = sizeof(double2) * (size_t)(n / 2 + 1) * ((ns + 1) / 2);
+  if (smem > 48 * 1024) return false;
+  const int th = ceil_div(lines, 128) < 152 * 2 ? 32 : 128;
+  const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(lines, th), (int64_t)152 * 32 * (128 / th));
+#define EFIE_FOLD(NH)                                                                                       \
+  if (half <= NH) {                                                                                         \
+    if (inverse) k_dft_inv_fold<NH><<<blocks, th, smem, s>>>(in, vin, out, vout, B, C, ax, e0, e1, e2, M, n); \
+    else k_dft_fwd_fold<NH><<<blocks, th, smem, s>>>(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n);   \
+    return true;                                                                                            \
+  }
+  EFIE_FOLD(4)
+  EFIE_FOLD(6)
+  EFIE_FOLD(10)
+#undef EFIE_FOLD
+  return false;
+}
+
 // Fused second and third passes (FP32, 32 channels), one block per
 // (box, x-frequency) slab.  Forward: the slab t[b][fx][y][z][c] (SP x SP x 32
 // values, the output of the x pass) is staged in shared memory; a warp takes
