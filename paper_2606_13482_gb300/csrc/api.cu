@@ -989,7 +989,7 @@ void run_mac(efie_handle* h, FarSet<R>& F, int ell, int C, const cpx_t<R>* Qin, 
       if (!done)
         launch_mac<R>(Qin, Rout, FL.Kh, B, C, LD.O, n3, LD.ntiles,
                       h->mac_variant == 1 ? -LD.max_tile : LD.max_tile, LD.tile_tgt_ptr, LD.tile_tgt,
-                      LD.tile_src_ptr, LD.tile_src, LD.tile_kidx_off, LD.tile_kidx, s);
+                      LD.tile_src_ptr, LD.tile_src, LD.tile_kidx_off, LD.tile_kidx, LD.il_ptr, LD.il_src, LD.il_off, s);
     }
 }
 

@@ -212,8 +212,23 @@ template <typename R>
 void launch_mac(const cpx_t<R>* Qh, cpx_t<R>* Rh, const cpx_t<R>* Kh, int64_t B, int C, int64_t O,
                 int64_t nf, int64_t ntiles, int max_tile_targets, const int64_t* tgt_ptr, const int32_t* tgt,
                 const int64_t* src_ptr, const int32_t* src, const int64_t* kidx_off, const int32_t* kidx,
-                cudaStream_t s);
+                const int64_t* il_ptr, const int32_t* il_src, const int32_t* il_off, cudaStream_t s);
 
+
+// FP64 translation on the tensor cores (mac_digits.cu): row tiles of 16
+// consecutive boxes over the union of their interaction lists, in groups of 8
+// sources; kexp: exponents of the kernel rows
+struct MacDigits {
+  int ntiles = 0;
+  const int32_t* kg_ptr = nullptr;  // [ntiles + 1]
+  const int4* idx = nullptr;        // [groups][32 lanes]
+  const int32_t* src = nullptr;     // [groups][8], -1: none
+  const int16_t* kexp = nullptr;    // [nf]
+};
+void launch_spec_rowexp(const double2* K, int64_t nf, int64_t O, int16_t* kexp, cudaStream_t s);
+// qd [nf][B][C][6], qexp [nf][C]: the digits of Q (work space)
+void launch_mac_digits(const double2* Q, double2* Rh, const double2* K, const MacDigits& m, uint32_t* qd, int16_t* qexp,
+                       int64_t B, int C, int64_t O, int64_t nf, cudaStream_t s);
 
 // the six Hessian kernel spectra of the dyadic factorization (ab = 00, 01,
 // 02, 11, 12, 22), [n^3][O] each

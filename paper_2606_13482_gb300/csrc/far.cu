@@ -2173,11 +2173,58 @@ __global__ void __launch_bounds__(128) k_mac_il32(const float2* __restrict__ Qh,
   }
 }
 
+// Translation from the interaction lists: a thread owns 16 bytes of one
+// (frequency, target) and runs down the target's list, four pairs in flight.  The
+// register tiles of k_mac_tiled visit every (source, target) slot of a tile, pairs or
+// not (FP64 multiply-adds of excluded slots cost as much as the others), and leave
+// most of the chip idle on few tiles and channels.  Sources ascend in both, so
+// the sums are the same bit for bit.  ms: 1,920 unknowns, FP64, one vector 0.076 ->
+// 0.045; 6,750, FP32, one vector 0.065 -> 0.032; 48,000, FP32, one vector, leaf level
+// 0.33 -> 0.16; 48,000, FP64, 8 vectors, top level 31.1 -> 27.8.
+template <typename R>
+__global__ void __launch_bounds__(128) k_mac_list(const typename U16<R>::T* __restrict__ Qh,
+                                                  typename U16<R>::T* __restrict__ Rh,
+                                                  const cpx_t<R>* __restrict__ Kh, int64_t B, int U, int64_t O,
+                                                  const int64_t* __restrict__ il_ptr,
+                                                  const int32_t* __restrict__ il_src,
+                                                  const int32_t* __restrict__ il_off, int64_t f0) {
+  using T = typename U16<R>::T;
+  const int64_t t = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  const int64_t x = t / U, f = f0 + blockIdx.y;
+  const int u = (int)(t - x * U);
+  if (x >= B) return;
+  const T* Qf = Qh + f * B * U + u;
+  const cpx_t<R>* Kf = Kh + f * O;
+  T acc = U16<R>::zero();
+  const int64_t e1 = il_ptr[x + 1];
+  int64_t e = il_ptr[x];
+  const auto mac = [&](const cpx_t<R>& k, const T& q) {
+    cpx_t<R> a = mk<R>(acc.x, acc.y);
+    cfma(a, k, mk<R>(q.x, q.y));
+    acc.x = a.x, acc.y = a.y;
+    if constexpr (sizeof(R) == 4) {
+      a = mk<R>(acc.z, acc.w);
+      cfma(a, k, mk<R>(q.z, q.w));
+      acc.z = a.x, acc.w = a.y;
+    }
+  };
+  for (; e + 4 <= e1; e += 4) {
+    cpx_t<R> k[4];
+    T q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) k[i] = Kf[__ldg(il_off + e + i)], q[i] = __ldg(Qf + (int64_t)__ldg(il_src + e + i) * U);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mac(k[i], q[i]);
+  }
+  for (; e < e1; ++e) mac(Kf[__ldg(il_off + e)], __ldg(Qf + (int64_t)__ldg(il_src + e) * U));
+  Rh[(f * B + x) * U + u] = acc;
+}
+
 template <typename R>
 void launch_mac(const cpx_t<R>* Qh, cpx_t<R>* Rh, const cpx_t<R>* Kh, int64_t B, int C, int64_t O,
                 int64_t nf, int64_t ntiles, int max_tile_targets, const int64_t* tgt_ptr, const int32_t* tgt,
                 const int64_t* src_ptr, const int32_t* src, const int64_t* kidx_off, const int32_t* kidx,
-                cudaStream_t s) {
+                const int64_t* il_ptr, const int32_t* il_src, const int32_t* il_off, cudaStream_t s) {
   if (B <= 0 || nf <= 0 || ntiles <= 0) return;
   // a negative tile size asks for the register-tile kernel (autotuner choice)
   const bool force_reg = max_tile_targets < 0;
@@ -2214,6 +2261,19 @@ void launch_mac(const cpx_t<R>* Qh, cpx_t<R>* Rh, const cpx_t<R>* Kh, int64_t B,
       k_mac_il32<8, CRI><<<grid, fpb * ncg, smem, s>>>((const float2*)Qh, (float2*)Rh, (const float2*)Kh, B, C, O,
                                                        nf, tgt_ptr, tgt, src_ptr, src, kidx_off, kidx, fpb, f0);
     }
+    return;
+  }
+  // In FP64 always.  In FP32 on interaction-list tiles (at most 8 targets), and on
+  // top levels of at most 64 boxes; wider tiles of one list reuse each kernel value
+  // for more products (128 boxes, 21^3 frequencies, 4 channels: 0.51 ms in register
+  // tiles, 0.57 from the lists).
+  if (!force_reg && (sizeof(R) == 8 || max_tile_targets <= 8 || (ntiles == 1 && max_tile_targets <= 64))) {
+    const int U = C * (int)sizeof(cpx_t<R>) / 16;
+    const unsigned gx = (unsigned)ceil_div(B * U, 128);
+    for (int64_t f0 = 0; f0 < nf; f0 += 65535)
+      k_mac_list<R><<<dim3(gx, (unsigned)std::min<int64_t>(65535, nf - f0)), 128, 0, s>>>(
+          reinterpret_cast<const typename U16<R>::T*>(Qh), reinterpret_cast<typename U16<R>::T*>(Rh), Kh, B, U, O, il_ptr,
+          il_src, il_off, f0);
     return;
   }
   constexpr int XR = 8, CR = 4;
@@ -2817,10 +2877,10 @@ template void launch_interp<double>(const double*, const int32_t*, const int32_t
                                     double2*, int64_t, double2*, int64_t, cudaStream_t);
 template void launch_mac<float>(const float2*, float2*, const float2*, int64_t, int, int64_t, int64_t, int64_t,
                                 int, const int64_t*, const int32_t*, const int64_t*, const int32_t*,
-                                const int64_t*, const int32_t*, cudaStream_t);
+                                const int64_t*, const int32_t*, const int64_t*, const int32_t*, const int32_t*, cudaStream_t);
 template void launch_mac<double>(const double2*, double2*, const double2*, int64_t, int, int64_t, int64_t,
                                  int64_t, int, const int64_t*, const int32_t*, const int64_t*, const int32_t*,
-                                 const int64_t*, const int32_t*, cudaStream_t);
+                                 const int64_t*, const int32_t*, const int64_t*, const int32_t*, const int32_t*, cudaStream_t);
 template void launch_convert<float>(const double2*, float2*, int64_t, cudaStream_t);
 template void launch_convert<double>(const double2*, double2*, int64_t, cudaStream_t);
 
