@@ -1724,9 +1724,11 @@ void launch_anterp(const R* gr, const R* gt, const int32_t* gptr_r, const int32_
 // ---------------------------------------------------------------- interpolation
 // yA[r][i] = sum_e sum_d m_d[e] r[b][pt(e)][d nr + r] for RWG i, and
 // u[r][t] = sum_e m^phi[e] r[b][pt(e)][3 nr + r] for triangle t (FP64
-// outputs).  One warp per basis function.  RWG: lane = channel d nr + r of
-// the vector part (3 nr <= 24 lanes), so every grid point is one coalesced
-// read; the three components are summed by shuffles at the end.  Triangle:
+// outputs).  RWG: lane = channel d nr + r of the vector part (3 nr <= 24 lanes),
+// so every grid point is one coalesced read; the three components are summed by
+// shuffles at the end.  A warp takes up to 32 / (3 nr) RWGs, `per` (21,870 RWGs, 3
+// right-hand sides of a chunk: 0.73 -> 0.64 ms with 3 of them; few RWGs keep one
+// per warp, for the latency of its loads).  Triangle:
 // the charge part is nr values per point, so the warp takes 32/nr entries at
 // a time, lane = (entry slot, r).
 template <typename R>
@@ -1740,23 +1742,23 @@ __global__ void __launch_bounds__(256) k_interp(const R* __restrict__ mr, const 
                                                 const int32_t* __restrict__ tri_box, int64_t Nt,
                                                 const cpx_t<R>* __restrict__ rg, int sp, int nr,
                                                 double2* __restrict__ yA, int64_t ldy, double2* __restrict__ u,
-                                                int64_t ldu) {
+                                                int64_t ldu, int per) {
   using T = cpx_t<R>;
   const int lane = threadIdx.x & 31;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= N + Nt) return;
+  const int64_t nw = (N + per - 1) / per;
+  if (w >= nw + Nt) return;
   const int npts = sp * sp * sp, C = 4 * nr;
   T acc = mk<R>(0, 0);
-  if (w < N) {
-    const int64_t i = w;
-    const int b0 = mr_base[3 * i], b1 = mr_base[3 * i + 1], b2 = mr_base[3 * i + 2];
-    const int e0 = mr_ext[3 * i], e1 = mr_ext[3 * i + 1], e2 = mr_ext[3 * i + 2];
-    const int ne = e0 * e1 * e2;
-    const bool act = lane < 3 * nr;
-    const int d = act ? lane / nr : 0;
-    const R* m = mr + mr_off[i] + d;  // entry e at m[3 e]
-    const T* gp = rg + (int64_t)rwg_box[i] * npts * C + lane;
-    if (act && ne > 0) {
+  if (w < nw) {
+    const int slot = lane / (3 * nr), ch = lane - slot * 3 * nr;
+    const int64_t i = w * per + slot;
+    const bool act = slot < per && i < N;
+    if (act) {
+      const int b0 = mr_base[3 * i], b1 = mr_base[3 * i + 1], b2 = mr_base[3 * i + 2];
+      const int e0 = mr_ext[3 * i], e1 = mr_ext[3 * i + 1], e2 = mr_ext[3 * i + 2];
+      const R* m = mr + mr_off[i] + ch / nr;  // entry e at m[3 e]
+      const T* gp = rg + (int64_t)rwg_box[i] * npts * C + ch;
       int e = 0;
       for (int a0 = 0; a0 < e0; ++a0)
         for (int a1 = 0; a1 < e1; ++a1) {
@@ -1774,9 +1776,9 @@ __global__ void __launch_bounds__(256) k_interp(const R* __restrict__ mr, const 
     }
     R sx = acc.x + __shfl_down_sync(0xffffffffu, acc.x, nr) + __shfl_down_sync(0xffffffffu, acc.x, 2 * nr);
     R sy = acc.y + __shfl_down_sync(0xffffffffu, acc.y, nr) + __shfl_down_sync(0xffffffffu, acc.y, 2 * nr);
-    if (lane < nr) yA[lane * ldy + i] = make_double2((double)sx, (double)sy);
+    if (act && ch < nr) yA[ch * ldy + i] = make_double2((double)sx, (double)sy);
   } else {
-    const int64_t i = w - N;
+    const int64_t i = w - nw;
     const int b0 = mt_base[3 * i], b1 = mt_base[3 * i + 1], b2 = mt_base[3 * i + 2];
     const int e0 = mt_ext[3 * i], e1 = mt_ext[3 * i + 1], e2 = mt_ext[3 * i + 2];
     const int ne = e0 * e1 * e2;
@@ -1934,10 +1936,12 @@ void launch_interp(const R* mr, const int32_t* mr_base, const int32_t* mr_ext, c
       return;
     }
   }
-  int64_t warps = N + Nt;
+  // RWGs per warp: as many as it has lanes for, while 32 warps per SM are left
+  const int per = (int)std::max<int64_t>(1, std::min<int64_t>(32 / (3 * nr), N / (152 * 32)));
+  int64_t warps = ceil_div(N, per) + Nt;
   int64_t blocks = ceil_div(warps * 32, 256);
   k_interp<R><<<(unsigned)blocks, 256, 0, s>>>(mr, mr_base, mr_ext, mr_off, rwg_box, N, mt, mt_base, mt_ext,
-                                               mt_off, tri_box, Nt, r, sp, nr, yA, ldy, u, ldu);
+                                               mt_off, tri_box, Nt, r, sp, nr, yA, ldy, u, ldu, per);
 }
 
 // ---------------------------------------------------------------- translation MAC
