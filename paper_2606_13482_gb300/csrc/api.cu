@@ -259,6 +259,7 @@ struct efie_handle {
   ~efie_handle() {
     if (net) efie::nn_delete(net);
     if (err_host) cudaFreeHost(err_host);
+    if (pin) cudaFreeHost(pin);
     if (ev_fork) cudaEventDestroy(ev_fork);
     if (ev_join) cudaEventDestroy(ev_join);
     if (ev_far) cudaEventDestroy(ev_far);
@@ -342,6 +343,8 @@ struct efie_handle {
   NearMma nmA = {}, nmS = {};
   int64_t nkgA = 0, nkgS = 0;
   int dig_ntt = 0;
+  void* pin = nullptr;    // page-locked landing place of the solver's coefficients
+  size_t pin_bytes = 0;
   int max_tset = 0;       // triangles of the largest leaf's triangle set
   // counts the (re)allocations of buffers that captured products refer to
   int64_t buf_gen = 0;
@@ -1850,18 +1853,23 @@ int solve_impl(efie_handle* h, const double2* b, double2* x, int n_rhs, double t
   std::vector<int> pc_fallback(n_rhs, 0);
   double2* wv = ws.take<double2>((int64_t)n_rhs * N);
   double2* rv = ws.take<double2>((int64_t)n_rhs * N);
-  double2* dh = ws.take<double2>((int64_t)n_rhs * (m + 1));
-  double2* dh2 = ws.take<double2>((int64_t)n_rhs * (m + 1));
-  double* dn = ws.take<double>(n_rhs);
+  // dh, dh2 and dn next to each other: one copy and one wait per iteration
+  double2* dh = ws.take<double2>((int64_t)2 * n_rhs * (m + 1) + (n_rhs + 1) / 2);
+  double* dn = reinterpret_cast<double*>(dh + (int64_t)2 * n_rhs * (m + 1));
+  const size_t pin_bytes = sizeof(double2) * (2 * (size_t)n_rhs * (m + 1) + (n_rhs + 1) / 2);
+  if (h->pin_bytes < pin_bytes) {
+    if (h->pin) cudaFreeHost(h->pin);
+    h->pin = nullptr;
+    h->pin_bytes = 0;
+    cuda_check(cudaHostAlloc(&h->pin, pin_bytes, cudaHostAllocDefault), "cudaHostAlloc");
+    h->pin_bytes = pin_bytes;
+  }
+  const std::complex<double>* pin = static_cast<const std::complex<double>*>(h->pin);
   int* dact = ws.take<int>(n_rhs);
   const int64_t ldr = (int64_t)(m + 1) * N;
   std::vector<double> bnorm(n_rhs), nrm(n_rhs);
   std::vector<int> its(n_rhs, 0), conv(n_rhs, 0), act(n_rhs, 1);
-  std::vector<std::complex<double>> hh((size_t)n_rhs * (m + 1)), hh2((size_t)n_rhs * (m + 1));
-  auto d2h = [&](std::vector<std::complex<double>>& dst, const double2* src, int64_t n) {
-    cuda_check(cudaMemcpyAsync(dst.data(), src, sizeof(double2) * n, cudaMemcpyDeviceToHost, s), "d2h");
-    cuda_check(cudaStreamSynchronize(s), "sync");
-  };
+  std::vector<std::complex<double>> hh(n_rhs);
   auto norms = [&](const double2* v, int64_t ld, std::vector<double>& out) {
     launch_norms(v, ld, N, n_rhs, dn, s);
     cuda_check(cudaMemcpyAsync(out.data(), dn, sizeof(double) * n_rhs, cudaMemcpyDeviceToHost, s), "d2h");
@@ -1938,15 +1946,18 @@ int solve_impl(efie_handle* h, const double2* b, double2* x, int n_rhs, double t
       KScope ks(h, K_KRYLOV, s, 5);
       launch_multidot(Vb, ldr, N, k + 1, wv, N, N, n_rhs, dact, dh, s);
       launch_multiaxpy(Vb, ldr, N, k + 1, dh, k + 1, wv, N, N, n_rhs, dact, -1.0, s);
-      launch_multidot(Vb, ldr, N, k + 1, wv, N, N, n_rhs, dact, dh2, s);
-      launch_multiaxpy(Vb, ldr, N, k + 1, dh2, k + 1, wv, N, N, n_rhs, dact, -1.0, s);
-      d2h(hh, dh, (int64_t)n_rhs * (k + 1));
-      d2h(hh2, dh2, (int64_t)n_rhs * (k + 1));
-      norms(wv, N, nrm);
+      const int64_t nc = (int64_t)n_rhs * (k + 1);
+      launch_multidot(Vb, ldr, N, k + 1, wv, N, N, n_rhs, dact, dh + nc, s);
+      launch_multiaxpy(Vb, ldr, N, k + 1, dh + nc, k + 1, wv, N, N, n_rhs, dact, -1.0, s);
+      launch_norms(wv, N, N, n_rhs, reinterpret_cast<double*>(dh + 2 * nc), s);
+      cuda_check(cudaMemcpyAsync(h->pin, dh, sizeof(double2) * 2 * nc + sizeof(double) * n_rhs,
+                                 cudaMemcpyDeviceToHost, s), "d2h");
+      cuda_check(cudaStreamSynchronize(s), "sync");
+      for (int r = 0; r < n_rhs; ++r) nrm[r] = std::sqrt(reinterpret_cast<const double*>(pin + 2 * nc)[r]);
       std::vector<std::complex<double>> sc((size_t)n_rhs, 0.0);
       for (int r = 0; r < n_rhs; ++r) {
         if (!inner[r]) continue;
-        for (int i = 0; i <= k; ++i) H[r][(size_t)i * m + k] = hh[(size_t)r * (k + 1) + i] + hh2[(size_t)r * (k + 1) + i];
+        for (int i = 0; i <= k; ++i) H[r][(size_t)i * m + k] = pin[r * (k + 1) + i] + pin[nc + r * (k + 1) + i];
         H[r][(size_t)(k + 1) * m + k] = nrm[r];
         sc[r] = nrm[r] > 0 ? 1.0 / nrm[r] : 0.0;
         // Givens: G = [[conj(c), conj(s)], [-s, c]], c = a/den, s = b/den

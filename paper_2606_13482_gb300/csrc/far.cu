@@ -2768,7 +2768,18 @@ __global__ void k_multiaxpy(const double2* __restrict__ Vb, int64_t ldv_r, int64
     int64_t r = idx / N, n = idx - r * N;
     if (active && !active[r]) continue;
     double2 acc = make_double2(0, 0);
-    for (int i = 0; i < nbasis; ++i) cfma(acc, h[r * hstride + i], Vb[r * ldv_r + i * ldv_i + n]);
+    // eight basis vectors in flight, summed in order
+    const double2* v = Vb + r * ldv_r + n;
+    const double2* hr = h + r * hstride;
+    int i = 0;
+    for (; i + 8 <= nbasis; i += 8) {
+      double2 b[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) b[q] = v[(i + q) * ldv_i];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) cfma(acc, hr[i + q], b[q]);
+    }
+    for (; i < nbasis; ++i) cfma(acc, hr[i], v[i * ldv_i]);
     double2 t = w[r * ldw + n];
     w[r * ldw + n] = make_double2(t.x + sign * acc.x, t.y + sign * acc.y);
   }
@@ -2778,9 +2789,10 @@ void launch_multiaxpy(const double2* Vb, int64_t ldv_r, int64_t ldv_i, int nbasi
                       double sign, cudaStream_t s) {
   int64_t total = N * nr;
   if (total <= 0 || nbasis <= 0) return;
-  int64_t blocks = ceil_div(total, 256);
+  const int th = total < 152 * 512 ? 64 : 256;  // short vectors over all SMs
+  int64_t blocks = ceil_div(total, th);
   if (blocks > 152 * 64) blocks = 152 * 64;
-  k_multiaxpy<<<(unsigned)blocks, 256, 0, s>>>(Vb, ldv_r, ldv_i, nbasis, h, hstride, w, ldw, N, nr, active,
+  k_multiaxpy<<<(unsigned)blocks, th, 0, s>>>(Vb, ldv_r, ldv_i, nbasis, h, hstride, w, ldw, N, nr, active,
                                                sign);
 }
 
