@@ -104,7 +104,9 @@ typedef struct {
     int64_t near_nnz_A, near_nnz_V;  /* near entries of A and of the scalar part (V on triangle
                                        pairs; Phi on A's RWG pairs for a direct-factorization
                                        handle) */
-    int64_t device_bytes;    /* estimated resident device bytes of the setup products */
+    int64_t device_bytes;    /* estimated resident device bytes of the setup products; for a
+                                handle, its device memory without the buffers that only make
+                                products faster and are given back when memory runs short */
     int64_t moment_entries_rwg;  /* leaf moment entries of all RWGs, per vector component */
     int64_t moment_entries_tri;  /* leaf moment entries of the scalar part: triangles (star),
                                     RWG divergences (direct handle) */
@@ -380,7 +382,8 @@ int efie_precond_gradient(efie_handle *h, const void *r, const void *e, float *g
  * frequency; 4: as 0 with the interaction-list levels of chunk pairs on CUDA
  * cores; 5: as 0 with a persistent form whose loader warp stages index
  * blocks, source spectra and kernel rows in shared memory by asynchronous
- * copies) and, for
+ * copies; FP64 passes run on tensor cores with 10-bit FP16 digits for every
+ * choice but 1) and, for
  * mixed handles, each near-field kernel (0: tensor cores, every operand cut
  * into 10-bit digits whose FP16 products are summed exactly; 1 to 3:
  * double-float arithmetic, with the source values 1: read through L1 with no

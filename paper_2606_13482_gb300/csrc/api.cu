@@ -137,6 +137,11 @@ struct FarSet {
   int Rc = 0;
   std::vector<cpx_t<R>*> q, r;
   cpx_t<R>*tmp1 = nullptr, *tmp2 = nullptr, *Qh = nullptr, *Rh = nullptr;
+  // FP64: digits of the source spectra of the largest level for chunks of up to
+  // Rc right-hand sides, and their exponents (optional: without them the
+  // translations run in FP64 arithmetic)
+  uint32_t* qd = nullptr;
+  int16_t* qexp = nullptr;
   // second chunk of a chunk pair (one translation pass per level over 16
   // right-hand sides): its level grids q2[], r2[], and spectra buffers for its
   // sources (Qt2) and results (Rt2)
@@ -155,6 +160,7 @@ struct LevDev {
   int32_t* il_src = nullptr;
   int32_t* il_off = nullptr;
   int32_t* offsets = nullptr;
+  MacDigits md;   // row tiles of the FP64 tensor-core translation (optional)
   int64_t* parent = nullptr;
   int8_t* bits = nullptr;
   int64_t* child_ptr = nullptr;
@@ -628,6 +634,19 @@ void ensure_far_buffers(efie_handle* h, FarSet<R>& F, int Rc) {
   F.Qh = h->mem.alloc<cpx_t<R>>(smax);
   F.Rh = h->mem.alloc<cpx_t<R>>(smax);
   F.Rc = Rc;
+  if constexpr (sizeof(R) == 8) {
+    h->mem.release_optional(F.qd);
+    h->mem.release_optional(F.qexp);
+    int64_t nmax = 0, fmax = 0;
+    for (int ell = P.D; ell >= P.top; --ell)
+      if (h->lev[ell - P.top].md.ntiles) {
+        const int64_t n3 = (int64_t)P.L(ell).nfft * P.L(ell).nfft * P.L(ell).nfft;
+        nmax = std::max(nmax, (int64_t)P.L(ell).code.size() * n3);
+        fmax = std::max(fmax, n3);
+      }
+    F.qd = nmax ? h->mem.alloc_optional<uint32_t>(nmax * C * 6) : nullptr;
+    F.qexp = F.qd ? h->mem.alloc_optional<int16_t>(fmax * C) : nullptr;
+  }
 }
 
 void ensure_work(efie_handle* h, int Rw) {
@@ -674,10 +693,27 @@ void drop_digits(efie_handle* h) {
   A.xexp = S.xexp = nullptr;
 }
 
-// gives back everything that only the tensor-core near field needs; products
-// run on the other near kernels from then on
+// the digits of the FP64 spectra, and the translation's tables
+void drop_mac_digits(efie_handle* h) {
+  if (h->f64.qd) ++h->buf_gen;
+  h->mem.release_optional(h->f64.qd);
+  h->mem.release_optional(h->f64.qexp);
+  h->f64.qd = nullptr;
+  h->f64.qexp = nullptr;
+  for (LevDev& L : h->lev) {
+    h->mem.release_optional(const_cast<int32_t*>(L.md.kg_ptr));
+    h->mem.release_optional(const_cast<int4*>(L.md.idx));
+    h->mem.release_optional(const_cast<int32_t*>(L.md.src));
+    h->mem.release_optional(const_cast<int16_t*>(L.md.kexp));
+    L.md = MacDigits();
+  }
+}
+
+// gives back everything that only the tensor-core near field and the FP64
+// tensor-core translation need; products run on the other kernels from then on
 void drop_near_mma(efie_handle* h) {
   drop_digits(h);
+  drop_mac_digits(h);
   for (NearMma* m : {&h->nmA, &h->nmS}) {
     h->mem.release_optional(const_cast<int64_t*>(m->rexp_off));
     h->mem.release_optional(const_cast<int64_t*>(m->kg_off));
@@ -818,6 +854,17 @@ void anterp_up(efie_handle* h, FarSet<R>& F, int nr, int rhs0, std::vector<cpx_t
   }
 }
 
+// one transform pass: folded (FP64), or with the conjugate pairing; false when
+// neither takes it
+template <typename R, typename FL_>
+bool dft_pass(const FL_& FL, const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, int64_t B, int C, int ax, int nin,
+              int e0, int e1, int e2, int n, bool inverse, cudaStream_t s) {
+  const cpx_t<R>* M = inverse ? FL.Mb : FL.Mf;
+  if constexpr (sizeof(R) == 8)
+    if (FL.folded && launch_dft_fold(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n, inverse, s)) return true;
+  return launch_dft<R>(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n, inverse, s);
+}
+
 template <typename R>
 void fwd_level(efie_handle* h, FarSet<R>& F, int ell, int C, const cpx_t<R>* qin, cpx_t<R>* Qout, cudaStream_t s) {
   Plan& P = h->plan;
@@ -844,17 +891,6 @@ void fwd_level(efie_handle* h, FarSet<R>& F, int ell, int C, const cpx_t<R>* qin
     launch_mode<R>(F.tmp1, a1, F.tmp2, a2, B, C, 1, sp, n, n, sp, FL.Mf, FL.Mf, true, nullptr, nullptr, false, s);
   if (!dft_pass<R>(FL, F.tmp2, a2, Qout, vf, B, C, 2, sp, n, n, n, n, false, s))
     launch_mode<R>(F.tmp2, a2, Qout, vf, B, C, 2, sp, n, n, n, FL.Mf, FL.Mf, true, nullptr, nullptr, false, s);
-}
-
-// one transform pass: folded (FP64), or with the conjugate pairing; false when
-// neither takes it
-template <typename R, typename FL_>
-bool dft_pass(const FL_& FL, const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, int64_t B, int C, int ax, int nin,
-              int e0, int e1, int e2, int n, bool inverse, cudaStream_t s) {
-  const cpx_t<R>* M = inverse ? FL.Mb : FL.Mf;
-  if constexpr (sizeof(R) == 8)
-    if (FL.folded && launch_dft_fold(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n, inverse, s)) return true;
-  return launch_dft<R>(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n, inverse, s);
 }
 
 template <typename R>
@@ -989,6 +1025,14 @@ void run_mac(efie_handle* h, FarSet<R>& F, int ell, int C, const cpx_t<R>* Qin, 
                                  LD.ntiles, LD.max_tile, LD.tile_tgt_ptr, LD.tile_tgt, LD.tile_src_ptr, LD.tile_src,
                                  LD.tile_kidx_off, LD.tile_kidx, h->err_dev, s);
       if (done) cuda_check(cudaPeekAtLastError(), "top-level translation (tensor-core kernel)");
+      if constexpr (sizeof(R) == 8)
+        // (4 channels of a few thousand tiles: the lists are faster, 0.045 ms against
+        // 0.053 for 1,920 unknowns)
+        if (LD.md.ntiles && F.qexp && h->mac_variant != 1 && (C > 4 || LD.md.ntiles * n3 >= 152 * 32)) {
+          launch_mac_digits(Qin, Rout, FL.Kh, LD.md, F.qd, F.qexp, B, C, LD.O, n3, s);
+          ks.launches(1);
+          done = true;
+        }
       if (!done)
         launch_mac<R>(Qin, Rout, FL.Kh, B, C, LD.O, n3, LD.ntiles,
                       h->mac_variant == 1 ? -LD.max_tile : LD.max_tile, LD.tile_tgt_ptr, LD.tile_tgt,
@@ -1296,6 +1340,62 @@ void do_matvec(efie_handle* h, const double2* x, int64_t ldx, double2* y, double
       matvec_chunk<double>(h, h->f64, x + (int64_t)(r0 - nr) * ldx, ldx, nr, yy, ya, yv, ldy, s);
   }
   cuda_check(cudaGetLastError(), "matvec launch");
+}
+
+// Tables of the FP64 tensor-core translation, level by level (left out where
+// the memory limit has no room for them).
+void build_mac_digits(efie_handle* h, cudaStream_t s) {
+  Plan& P = h->plan;
+  for (int ell = P.D; ell >= P.top; --ell) {
+    const Level& L = P.L(ell);
+    LevDev& LD = h->lev[ell - P.top];
+    if (LD.nfar == 0) continue;
+    const int64_t B = (int64_t)L.code.size(), n3 = (int64_t)L.nfft * L.nfft * L.nfft;
+    std::vector<int32_t> kg(1, 0), src, pos(B, -1), un;
+    std::vector<int32_t> idx;  // [group][lane][4]
+    for (int64_t x0 = 0; x0 < B; x0 += 16) {
+      const int64_t x1 = std::min<int64_t>(B, x0 + 16);
+      un.clear();
+      for (int64_t e = L.il_ptr[x0]; e < L.il_ptr[x1]; ++e) un.push_back(L.il_src[e]);
+      std::sort(un.begin(), un.end());
+      un.erase(std::unique(un.begin(), un.end()), un.end());
+      const size_t ng = (un.size() + 7) / 8, i0 = idx.size();
+      idx.resize(i0 + ng * 128, -1);
+      src.resize(src.size() + ng * 8, -1);
+      std::copy(un.begin(), un.end(), src.end() - (int64_t)(ng * 8));
+      for (size_t i = 0; i < un.size(); ++i) pos[un[i]] = (int32_t)i;
+      // lane 4 g + t of a group holds (row g, source t), (g + 8, t), (g, t + 4), (g + 8, t + 4)
+      for (int64_t x = x0; x < x1; ++x)
+        for (int64_t e = L.il_ptr[x]; e < L.il_ptr[x + 1]; ++e) {
+          const int p = pos[L.il_src[e]], c = p & 7, r = (int)(x - x0);
+          idx[i0 + (size_t)(p >> 3) * 128 + (size_t)(4 * (r & 7) + (c & 3)) * 4 + (r >> 3) + 2 * (c >> 2)] = L.il_off[e];
+        }
+      kg.push_back(kg.back() + (int32_t)ng);
+    }
+    DevMem& M = h->mem;
+    const auto up = [&](const auto& v) {
+      using T = typename std::decay<decltype(v[0])>::type;
+      T* d = M.alloc_optional<T>((int64_t)v.size());
+      if (d && !v.empty())
+        cuda_check(cudaMemcpy(d, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice), "translation tables");
+      return d;
+    };
+    MacDigits m;
+    m.kg_ptr = up(kg);
+    m.idx = reinterpret_cast<const int4*>(up(idx));
+    m.src = up(src);
+    int16_t* ke = M.alloc_optional<int16_t>(n3);
+    m.kexp = ke;
+    if (m.kg_ptr && m.idx && m.src && ke) {
+      launch_spec_rowexp(h->f64.lv[ell - P.top].Kh, n3, LD.O, ke, s);
+      m.ntiles = (int)kg.size() - 1;
+    }
+    LD.md = m;
+    if (!m.ntiles) {
+      drop_mac_digits(h);
+      return;
+    }
+  }
 }
 
 // ------------------------------------------------------------- setup
@@ -1801,6 +1901,7 @@ void setup_impl(efie_handle* h, const efie_mesh* mesh, double k, int p, double g
   build_far<double>(h, h->f64, s);
   std::vector<double2*> K64 = build_kernel_spectra64(h, s);
   build_spectra<double>(h, h->f64, K64, s);
+  build_mac_digits(h, s);
   if (h->precision == EFIE_MIXED) {
     build_far<float>(h, h->f32, s);
     build_spectra<float>(h, h->f32, K64, s);
@@ -2493,7 +2594,7 @@ int efie_num_unknowns(const efie_handle* h, int64_t* n) {
 int efie_plan_info(const efie_handle* h, efie_plan_info_t* info) {
   if (!h || !info) return EFIE_EINVAL;
   fill_plan_info(h->plan, info, nullptr, 0);
-  info->device_bytes = h->mem.bytes;
+  info->device_bytes = h->mem.bytes - h->mem.optional_bytes;
   if (h->direct) {
     // the scalar part is Phi on the RWG pairs of the A blocks, its moments per RWG
     info->near_nnz_V = info->near_nnz_A;

@@ -157,12 +157,6 @@ bool dft_yz_fits(int sp, int n);   // the fused forward pass takes this level
 bool dft_zy_fits(int sp, int n);   // the fused inverse pass takes this level
 
 
-// DFT passes of the stabilized transforms using the conjugate symmetry of
-// M = F P (forward, n x nin) / P^T F^{-1} (inverse, nout x n); false when no
-// specialisation fits
-template <typename R>
-bool launch_dft(const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, int64_t B, int C, int ax, int nin,
-                int e0, int e1, int e2, const cpx_t<R>* M, int n, bool inverse, cudaStream_t s);
 
 // top grid level on the tensor cores (tcgen05, kind::tf32 with a 3-term split,
 // FP32-class products); false when the configuration does not fit it
