@@ -214,7 +214,7 @@ static bool dispatch_mode_line(const cpx_t<R>* in, View vin, cpx_t<R>* out, View
 // output, which read every input nout times and every matrix value from L1 (k_mode),
 // and register-resident lines of up to 40 values, which spilled.  On a nonuniform
 // tree with 32 boxes of 41^3 splines (77 frequencies per axis) and 52 of 25^3, 64
-// vectors, ms: forward 333 -> 69, inverse 437 -> 69, upward 181 -> 11, downward
+// vectors, ms: forward 333 -> 62, inverse 437 -> 63 (with k_mode_tile2 below), upward 181 -> 11, downward
 // 27 -> 7.  Up to 21 inputs the register-resident line kernels stay: there the
 // passes run near the memory bandwidth.
 template <int MODE>
@@ -413,10 +413,199 @@ __global__ void __launch_bounds__(320) k_mode_tile(const cpx_t<R>* __restrict__ 
   }
 }
 
+// The FP32 complex and paired passes (MODE 1 and 2) with two units (four lines)
+// per lane: a broadcast matrix value feeds four lines instead of two, which
+// halves the shared-memory returns per multiply-add.  The sums of JT outputs of
+// four lines stay in registers (up to 168: twelve warps per SM, whatever the
+// block size BT), a warp owns one tile of JT outputs, and the inputs come in
+// pieces of 16 through a ring of three, so that three blocks of four warps fit on
+// an SM with their matrices.  Same sums in the same order as k_mode_tile.
+//
+// What bounds it: issue slots (three quarters taken, four fifths of them
+// multiply-adds; register-bank conflicts take most of the others).  41 -> 77
+// complex outputs, 64 vectors, 32 boxes of 77 x 77 lines: 3.93 -> 3.59 ms; the
+// transforms of that tree: forward 68.7 -> 62.1, inverse 69.1 -> 63.4 ms.  Reading
+// the next input's values ahead by hand changed nothing.
+constexpr int T2_PI = 16, T2_RD = 3;
+template <int MODE, int JT, int BT>
+__global__ void __launch_bounds__(BT, 384 / BT) k_mode_tile2(const float2* __restrict__ in, float2* __restrict__ out,
+                                                             const TileArgs<MODE> a) {
+  extern __shared__ __align__(16) unsigned char tile_smem[];
+  const int nj = MODE == 2 ? a.n / 2 + 1 : a.nout;
+  const int njt = (nj + JT - 1) / JT;
+  constexpr int JP = JT + (JT & 1);  // matrix tile, padded to 16 bytes
+  const int msz = a.nin * njt * JP;
+  float2* Ms = reinterpret_cast<float2*>(tile_smem);               // [nin][njt][JP]
+  float4* ring = reinterpret_cast<float4*>(Ms + msz);              // [T2_RD][T2_PI][64]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+  for (int e = tid; e < msz; e += blockDim.x) {
+    const int i = e / (njt * JP), q = e - i * (njt * JP), jt = q / JP, jl = q - jt * JP, j = jt * JT + jl;
+    Ms[e] = jl < JT && j < nj ? reinterpret_cast<const float2*>(a.M0)[(int64_t)j * a.nin + i] : make_float2(0.f, 0.f);
+  }
+  const int CL = a.C / 2, units = a.ea * a.eb * CL;
+  const int64_t sa_in = a.ax == 0 ? a.vin.s1 : a.vin.s0, sb_in = a.ax == 2 ? a.vin.s1 : a.vin.s2;
+  const int64_t sa_out = a.ax == 0 ? a.vout.s1 : a.vout.s0, sb_out = a.ax == 2 ? a.vout.s1 : a.vout.s2;
+  const int64_t step_in = a.ax == 0 ? a.vin.s0 : (a.ax == 1 ? a.vin.s1 : a.vin.s2);
+  const int64_t step_out = a.ax == 0 ? a.vout.s0 : (a.ax == 1 ? a.vout.s1 : a.vout.s2);
+  // offset of unit 32 h + lane of an item in its box (-1: past the last)
+  auto offset = [&](int64_t item, int h, bool output) -> int64_t {
+    const int64_t b = item / a.ngrp;
+    const int u = (int)(item - b * a.ngrp) * 64 + 32 * h + lane;
+    if (u >= units) return -1;
+    const int c = (u % CL) * 2, t = u / CL, ib = t % a.eb, ia = t / a.eb;
+    return output ? b * a.vout.sb + ia * sa_out + ib * sb_out + c : b * a.vin.sb + ia * sa_in + ib * sb_in + c;
+  };
+  const int npc = (a.nin + T2_PI - 1) / T2_PI;
+  // loader: pieces of the block's items in order
+  int64_t litem = blockIdx.x, lo0 = -1, lo1 = -1;
+  int lpc = 0;
+  if (litem < a.items) lo0 = offset(litem, 0, false), lo1 = offset(litem, 1, false);
+  auto load = [&](int slot) {
+    if (litem < a.items) {
+      float4* d = ring + slot * (T2_PI * 64) + lane;
+      const int i0 = lpc * T2_PI, i1 = min(a.nin, i0 + T2_PI);
+      for (int i = i0 + warp; i < i1; i += nw) {
+        if (lo0 >= 0) tile_cp16(d + (i - i0) * 64, in + lo0 + i * step_in);
+        if (lo1 >= 0) tile_cp16(d + (i - i0) * 64 + 32, in + lo1 + i * step_in);
+      }
+      if (++lpc == npc) {
+        lpc = 0;
+        litem += gridDim.x;
+        if (litem < a.items) lo0 = offset(litem, 0, false), lo1 = offset(litem, 1, false);
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+#pragma unroll
+  for (int q = 0; q < T2_RD - 1; ++q) load(q);
+  int slot = 0;
+  constexpr int NA = MODE == 2 ? 4 : 2;  // sums per output and line
+  for (int64_t item = blockIdx.x; item < a.items; item += gridDim.x) {
+    float acc[JT][4][NA];
+#pragma unroll
+    for (int j = 0; j < JT; ++j)
+#pragma unroll
+      for (int l = 0; l < 4; ++l)
+#pragma unroll
+        for (int q = 0; q < NA; ++q) acc[j][l][q] = 0.f;
+    for (int pc = 0; pc < npc; ++pc) {
+      asm volatile("cp.async.wait_group %0;\n" ::"n"(T2_RD - 2) : "memory");
+      __syncthreads();  // this piece is in for every warp, and every warp has left the one before
+      load(slot == 0 ? T2_RD - 1 : slot - 1);
+      if (warp < njt) {
+        const float4* tp = ring + slot * (T2_PI * 64) + lane;
+        const int i0 = pc * T2_PI, cnt = min(T2_PI, a.nin - i0);
+        const float4* mp = reinterpret_cast<const float4*>(Ms + ((size_t)i0 * njt + warp) * JP);
+#pragma unroll 2
+        for (int i = 0; i < cnt; ++i) {
+          const float4 w0 = tp[i * 64], w1 = tp[i * 64 + 32];
+          const float2 v[4] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w), make_float2(w1.x, w1.y),
+                               make_float2(w1.z, w1.w)};
+          float2 m[JP];
+#pragma unroll
+          for (int q = 0; q < JP / 2; ++q) {
+            const float4 t = mp[(size_t)i * njt * (JP / 2) + q];
+            m[2 * q] = make_float2(t.x, t.y);
+            m[2 * q + 1] = make_float2(t.z, t.w);
+          }
+#pragma unroll
+          for (int j = 0; j < JT; ++j)
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+              if constexpr (MODE == 2) {
+                acc[j][l][0] = fmaf(m[j].x, v[l].x, acc[j][l][0]);
+                acc[j][l][1] = fmaf(m[j].y, v[l].y, acc[j][l][1]);
+                acc[j][l][2] = fmaf(m[j].x, v[l].y, acc[j][l][2]);
+                acc[j][l][3] = fmaf(m[j].y, v[l].x, acc[j][l][3]);
+              } else {
+                acc[j][l][0] = fmaf(m[j].x, v[l].x, acc[j][l][0]);
+                acc[j][l][0] = fmaf(-m[j].y, v[l].y, acc[j][l][0]);
+                acc[j][l][1] = fmaf(m[j].x, v[l].y, acc[j][l][1]);
+                acc[j][l][1] = fmaf(m[j].y, v[l].x, acc[j][l][1]);
+              }
+            }
+        }
+      }
+      slot = slot == T2_RD - 1 ? 0 : slot + 1;
+    }
+    if (warp < njt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int64_t o = offset(item, h, true);
+        if (o < 0) continue;
+        float2* op = out + o;
+#pragma unroll
+        for (int j = 0; j < JT; ++j) {
+          const int jo = warp * JT + j;
+          if (jo >= nj) break;
+          const float* p = acc[j][2 * h];
+          const float* q = acc[j][2 * h + 1];
+          if constexpr (MODE == 2) {
+            *reinterpret_cast<float4*>(op + jo * step_out) =
+                make_float4(p[0] - p[1], p[2] + p[3], q[0] - q[1], q[2] + q[3]);
+            if (jo != 0 && 2 * jo != a.n)
+              *reinterpret_cast<float4*>(op + (int64_t)(a.n - jo) * step_out) =
+                  make_float4(p[0] + p[1], p[2] - p[3], q[0] + q[1], q[2] - q[3]);
+          } else {
+            float4 r = make_float4(p[0], p[1], q[0], q[1]);
+            if (a.accumulate) {
+              const float4 old = *reinterpret_cast<const float4*>(op + jo * step_out);
+              r = make_float4(r.x + old.x, r.y + old.y, r.z + old.z, r.w + old.w);
+            }
+            *reinterpret_cast<float4*>(op + jo * step_out) = r;
+          }
+        }
+      }
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+}
+
+template <int MODE, int JT, int BT>
+static void run_mode_tile2_bt(const float2* in, float2* out, const TileArgs<MODE>& a, int warps, size_t smem,
+                              cudaStream_t s) {
+  const int bps = (int)std::max<size_t>(1, std::min<size_t>(220 * 1024 / (smem + 1024), 384 / BT));
+  static SmemAttr attr;
+  smem_attr_once(k_mode_tile2<MODE, JT, BT>, (int)smem, attr.v);
+  k_mode_tile2<MODE, JT, BT>
+      <<<(unsigned)std::min<int64_t>(a.items, (int64_t)152 * bps), 32 * warps, smem, s>>>(in, out, a);
+}
+template <int MODE, int JT>
+static bool run_mode_tile2(const float2* in, float2* out, int64_t B, TileArgs<MODE> a, cudaStream_t s) {
+  const int nj = MODE == 2 ? a.n / 2 + 1 : a.nout, njt = (nj + JT - 1) / JT;
+  const size_t smem = sizeof(float2) * (size_t)a.nin * njt * (JT + (JT & 1)) + (size_t)T2_RD * T2_PI * 64 * 16;
+  const int64_t units = (int64_t)a.ea * a.eb * (a.C / 2);
+  if (njt > 12 || smem > 200 * 1024 || units > 0x7fffffff - 64) return false;
+  a.ngrp = (int)((units + 63) / 64);
+  a.items = B * a.ngrp;
+  if (a.items <= 0) return true;
+  const int warps = std::max(njt, 4);  // spare warps help to load
+  if (warps <= 4) run_mode_tile2_bt<MODE, JT, 128>(in, out, a, warps, smem, s);
+  else if (warps <= 6) run_mode_tile2_bt<MODE, JT, 192>(in, out, a, warps, smem, s);
+  else run_mode_tile2_bt<MODE, JT, 384>(in, out, a, warps, smem, s);
+  return true;
+}
+
 // false when the matrix and two input buffers do not fit in shared memory, or
 // when a unit's 16 bytes would not be aligned (an odd channel count in FP32)
 template <typename R, int MODE>
 static bool launch_mode_tile(const cpx_t<R>* in, cpx_t<R>* out, int64_t B, TileArgs<MODE> a, cudaStream_t s) {
+  // FP32 complex passes: two units per lane, up to 12 tiles of outputs (84 to 96
+  // outputs, 144 paired ones); beyond that k_mode_tile, whose warps take several
+  // tiles in turn.  The tile that leaves less of its last one empty.
+  if constexpr (sizeof(R) == 4 && (MODE == 1 || MODE == 2)) {
+    if (a.C % 2 == 0 && !a.srcmap) {
+      const auto pad = [&](int nj, int jt) { return (nj + jt - 1) / jt * jt; };
+      if constexpr (MODE == 2) {
+        const int nj = a.n / 2 + 1;
+        if (pad(nj, 5) < pad(nj, 6) ? run_mode_tile2<MODE, 5>(in, out, B, a, s)
+                                    : run_mode_tile2<MODE, 6>(in, out, B, a, s))
+          return true;
+      } else if (pad(a.nout, 7) < pad(a.nout, 8) ? run_mode_tile2<MODE, 7>(in, out, B, a, s)
+                                                 : run_mode_tile2<MODE, 8>(in, out, B, a, s)) {
+        return true;
+      }
+    }
+  }
   constexpr int LPT = 16 / (int)sizeof(cpx_t<R>);
   constexpr bool CM = MODE == 1 || MODE == 2;
   if (a.C % LPT != 0) return false;

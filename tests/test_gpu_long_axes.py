@@ -1,4 +1,4 @@
-"""Mode products along long axes (the tiled kernel): a two-level tree with 23
+"""Mode products along long axes (the tiled kernels): a two-level tree with 23
 leaf splines per axis, so that the transforms take 27 and 47 splines, the upward
 transfer 27 -> 47 and the downward one 47 -> 27, for 1, 3 and 8 right-hand sides
 (4, 12 and 32 channels), against the oracle; and the anterpolation's lane forms
