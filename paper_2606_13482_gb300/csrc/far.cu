@@ -2702,8 +2702,8 @@ void launch_combine(const double2* yA, int64_t ldA, const double2* w, int64_t ld
                                              y, ldy, yAout, yVout);
 }
 
-// Plane-wave RHS: per RWG, both triangles with a degree-10 collapsed rule
-// (boxes with more than 1,472 triangles).
+// Plane-wave RHS: per RWG, both triangles with a degree-10 collapsed rule (up to
+// RHS_DIRECT waves, and boxes with more than 1,472 triangles).
 __constant__ double c_q6[3][36];
 __global__ void k_rhs_pw(const double* __restrict__ V, const int32_t* __restrict__ T,
                          const double* __restrict__ area, const int32_t* __restrict__ tri_pm,
@@ -2882,15 +2882,20 @@ int upload_rhs_rule(const double* q6) {
                   cudaMemcpyToSymbol(c_pw_s, sc, sizeof(sc)) == cudaSuccess;
   return ok ? 0 : -1;
 }
+constexpr int RHS_DIRECT = 64;
 void launch_rhs_planewave(const RhsGeom& g, const double* khat, const double* pol, int nr, double2* rhs, int64_t ld,
                           cudaStream_t s) {
   int64_t total = g.N * nr;
   if (total <= 0) return;
-  // by leaf box where its triangles' integrals fit in shared memory, up to 8
-  // waves at a time (46 KB: no opt-in, four blocks per SM)
+  // More waves than one chunk of a product has vectors: by leaf box where its
+  // triangles' integrals fit in shared memory, up to 8 waves at a time (46 KB: no
+  // opt-in, four blocks per SM).  65 waves, 58,080 unknowns: 22.9 ms direct, 2.4 by
+  // box.  Fewer waves keep every bit of the direct sums: they are what products and
+  // solves take as vectors, an FP32 product rounds them, and a last bit of a component
+  // on a rounding boundary moves that product by up to 3e-9.
   const int64_t per = 2 * sizeof(double2) * (int64_t)g.max_tset;
   const int W = (int)std::min<int64_t>(std::min(nr, 8), 46 * 1024 / std::max<int64_t>(per, 1));
-  if (W >= 1 && g.n_boxes > 0 && (nr + W - 1) / W <= 65535) {
+  if (nr > RHS_DIRECT && W >= 1 && g.n_boxes > 0 && (nr + W - 1) / W <= 65535) {
     k_rhs_box<<<dim3((unsigned)g.n_boxes, (unsigned)((nr + W - 1) / W)), 128, (size_t)(W * per), s>>>(g, khat, pol, nr,
                                                                                                   W, rhs, ld);
     return;
