@@ -1024,7 +1024,7 @@ __global__ void k_dft_fwd_line(const cpx_t<R>* __restrict__ in, View vin, cpx_t<
 
 // Inverse passes keep the nout (= s') outputs of a line in registers and
 // stream the conjugate input pairs (f, n - f) through them.
-template <typename R, int AMAX, int LPT>
+template <typename R, int AMAX>
 __global__ void k_dft_inv_line(const cpx_t<R>* __restrict__ in, View vin, cpx_t<R>* __restrict__ out, View vout,
                                int64_t B, int C, int ax, int nin_unused, int e0, int e1, int e2,
                                const cpx_t<R>* __restrict__ M, int n) {
@@ -1043,84 +1043,55 @@ __global__ void k_dft_inv_line(const cpx_t<R>* __restrict__ in, View vin, cpx_t<
   const int64_t sa_out = ax == 0 ? vout.s1 : vout.s0, sb_out = ax == 2 ? vout.s1 : vout.s2;
   const int64_t step_in = ax == 0 ? vin.s0 : (ax == 1 ? vin.s1 : vin.s2);
   const int64_t step_out = ax == 0 ? vout.s0 : (ax == 1 ? vout.s1 : vout.s2);
-  const int CL = C / LPT;
-  const int64_t lines = B * ea * eb * (int64_t)CL;
+  const int64_t lines = B * ea * eb * (int64_t)C;
   const int np = (n - 1) / 2;     // conjugate pairs (f, n - f), f = 1 .. np
   const bool mid = (n % 2) == 0;  // f = n/2 pairs with itself
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < lines;
        idx += (int64_t)gridDim.x * blockDim.x) {
     int64_t t = idx;
-    const int c = (int)(t % CL) * LPT;
-    t /= CL;
+    const int c = (int)(t % C);
+    t /= C;
     const int ib = (int)(t % eb);
     t /= eb;
     const int ia = (int)(t % ea);
     const int64_t b = t / ea;
     const T* ip = in + b * vin.sb + ia * sa_in + ib * sb_in + c;
-    T acc[AMAX][LPT];
+    T acc[AMAX];
     {
-      T v0[LPT];
-#pragma unroll
-      for (int l = 0; l < LPT; ++l) v0[l] = ip[l];
+      const T v0 = ip[0];
 #pragma unroll
       for (int a = 0; a < AMAX; ++a)
-        if (a < nout) {
-          const T m = Ms[a];
-#pragma unroll
-          for (int l = 0; l < LPT; ++l) acc[a][l] = cmul(m, v0[l]);
-        }
+        if (a < nout) acc[a] = cmul(Ms[a], v0);
     }
-    T z1[LPT], z2[LPT];
-#pragma unroll
-    for (int l = 0; l < LPT; ++l) {
-      z1[l] = np > 0 ? ip[step_in + l] : mk<R>(0, 0);
-      z2[l] = np > 0 ? ip[(int64_t)(n - 1) * step_in + l] : mk<R>(0, 0);
-    }
+    T z1 = np > 0 ? ip[step_in] : mk<R>(0, 0), z2 = np > 0 ? ip[(int64_t)(n - 1) * step_in] : mk<R>(0, 0);
     for (int f = 1; f <= np; ++f) {
-      T u[LPT], w[LPT];
-#pragma unroll
-      for (int l = 0; l < LPT; ++l) {
-        u[l] = mk<R>(z1[l].x + z2[l].x, z1[l].y + z2[l].y);
-        w[l] = mk<R>(z1[l].x - z2[l].x, z1[l].y - z2[l].y);
-      }
+      const T u = mk<R>(z1.x + z2.x, z1.y + z2.y), w = mk<R>(z1.x - z2.x, z1.y - z2.y);
       if (f < np) {  // next pair's loads in flight during this pair's products
-#pragma unroll
-        for (int l = 0; l < LPT; ++l) {
-          z1[l] = ip[(int64_t)(f + 1) * step_in + l];
-          z2[l] = ip[(int64_t)(n - f - 1) * step_in + l];
-        }
+        z1 = ip[(int64_t)(f + 1) * step_in];
+        z2 = ip[(int64_t)(n - f - 1) * step_in];
       }
       const T* Mr = Ms + f * nout;
 #pragma unroll
       for (int a = 0; a < AMAX; ++a)
         if (a < nout) {
           const T m = Mr[a];
-#pragma unroll
-          for (int l = 0; l < LPT; ++l) {
-            acc[a][l].x = fma(m.x, u[l].x, acc[a][l].x);
-            acc[a][l].x = fma(-m.y, w[l].y, acc[a][l].x);
-            acc[a][l].y = fma(m.x, u[l].y, acc[a][l].y);
-            acc[a][l].y = fma(m.y, w[l].x, acc[a][l].y);
-          }
+          acc[a].x = fma(m.x, u.x, acc[a].x);
+          acc[a].x = fma(-m.y, w.y, acc[a].x);
+          acc[a].y = fma(m.x, u.y, acc[a].y);
+          acc[a].y = fma(m.y, w.x, acc[a].y);
         }
     }
     if (mid) {
       const T* Mr = Ms + (n / 2) * nout;
-      T vm[LPT];
-#pragma unroll
-      for (int l = 0; l < LPT; ++l) vm[l] = ip[(int64_t)(n / 2) * step_in + l];
+      const T vm = ip[(int64_t)(n / 2) * step_in];
 #pragma unroll
       for (int a = 0; a < AMAX; ++a)
-        if (a < nout)
-#pragma unroll
-          for (int l = 0; l < LPT; ++l) cfma(acc[a][l], Mr[a], vm[l]);
+        if (a < nout) cfma(acc[a], Mr[a], vm);
     }
     T* op = out + b * vout.sb + ia * sa_out + ib * sb_out + c;
 #pragma unroll
     for (int a = 0; a < AMAX; ++a)
-      if (a < nout)
-#pragma unroll
-        for (int l = 0; l < LPT; ++l) op[a * step_out + l] = acc[a][l];
+      if (a < nout) op[a * step_out] = acc[a];
   }
 }
 
@@ -1297,10 +1268,13 @@ bool launch_dft_fold(const double2* in, View vin, double2* out, View vout, int64
 // into the spectrum layout Q[fx][fy][fz][b][c] (256 contiguous bytes per
 // warp store).  The y-pass intermediate never goes to HBM: per box the pass
 // pair reads n SP^2 and writes n^3 values instead of reading and writing
-// n SP^2 + n^2 SP.
+// n SP^2 + n^2 SP.  What bounds it: issue slots (two thirds taken) with HBM at
+// 4.5 TB/s.  508 boxes of 9^3 splines, 16 vectors: 215 -> 175 us (one matrix read per
+// row and a warp of eight idle before).
 template <int SP>
-__global__ void __launch_bounds__(256, 2) k_dft_fwd_yz(const float2* __restrict__ in, float2* __restrict__ out,
-                                                    int64_t B, const float2* __restrict__ M, int n) {
+__global__ void __launch_bounds__(256, SP == 9 ? 3 : 1)
+    k_dft_fwd_yz(const float2* __restrict__ in, float2* __restrict__ out, int64_t B, const float2* __restrict__ M,
+                 int n) {
   extern __shared__ float4 fyz_smem[];
   float2* slab = reinterpret_cast<float2*>(fyz_smem);  // [SP][SP][32]
   float2* Ms = slab + SP * SP * 32;                    // rows 0 .. n/2 of M, [f][SP]
@@ -1311,8 +1285,9 @@ __global__ void __launch_bounds__(256, 2) k_dft_fwd_yz(const float2* __restrict_
   {
     const float4* src = reinterpret_cast<const float4*>(in + sl * (SP * SP * 32));
     float4* dst = reinterpret_cast<float4*>(slab);
-    for (int i = threadIdx.x; i < SP * SP * 16; i += blockDim.x) dst[i] = src[i];
+    for (int i = threadIdx.x; i < SP * SP * 16; i += blockDim.x) tile_cp16(dst + i, src + i);
     for (int i = threadIdx.x; i < nh * SP; i += blockDim.x) Ms[i] = M[i];
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -1343,72 +1318,195 @@ __global__ void __launch_bounds__(256, 2) k_dft_fwd_yz(const float2* __restrict_
       t0[z] = make_float2(a.x - c.x, a.y + c.y);
       t1[z] = make_float2(a.x + c.x, a.y - c.y);
     }
+    // a matrix value serves both rows
+    float2* op = out + (((int64_t)fx * n + fy) * n * B + b) * 32 + lane;
+    float2* oq = out + (((int64_t)fx * n + (n - fy)) * n * B + b) * 32 + lane;
     const bool ypair = fy != 0 && 2 * fy != n;
-    for (int r = 0; r < (ypair ? 2 : 1); ++r) {
-      const int fyr = r == 0 ? fy : n - fy;
-      float2* op = out + (((int64_t)fx * n + fyr) * n * B + b) * 32 + lane;
-      for (int fz = 0; fz < nh; ++fz) {
-        const float2* Mz = Ms + fz * SP;
-        float s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f;
+    for (int fz = 0; fz < nh; ++fz) {
+      const float2* Mz = Ms + fz * SP;
+      const bool zpair = fz != 0 && 2 * fz != n;
+      float s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f, r1 = 0.f, r2 = 0.f, r3 = 0.f, r4 = 0.f;
 #pragma unroll
-        for (int z = 0; z < SP; ++z) {
-          const float2 m = Mz[z];
-          const float2 v = r == 0 ? t0[z] : t1[z];
-          s1 = fmaf(m.x, v.x, s1);
-          s2 = fmaf(m.y, v.y, s2);
-          s3 = fmaf(m.x, v.y, s3);
-          s4 = fmaf(m.y, v.x, s4);
-        }
-        op[fz * fstride] = make_float2(s1 - s2, s3 + s4);
-        if (fz != 0 && 2 * fz != n) op[(int64_t)(n - fz) * fstride] = make_float2(s1 + s2, s3 - s4);
+      for (int z = 0; z < SP; ++z) {
+        const float2 m = Mz[z];
+        s1 = fmaf(m.x, t0[z].x, s1);
+        s2 = fmaf(m.y, t0[z].y, s2);
+        s3 = fmaf(m.x, t0[z].y, s3);
+        s4 = fmaf(m.y, t0[z].x, s4);
+        r1 = fmaf(m.x, t1[z].x, r1);
+        r2 = fmaf(m.y, t1[z].y, r2);
+        r3 = fmaf(m.x, t1[z].y, r3);
+        r4 = fmaf(m.y, t1[z].x, r4);
+      }
+      op[fz * fstride] = make_float2(s1 - s2, s3 + s4);
+      if (zpair) op[(int64_t)(n - fz) * fstride] = make_float2(s1 + s2, s3 - s4);
+      if (ypair) {
+        oq[fz * fstride] = make_float2(r1 - r2, r3 + r4);
+        if (zpair) oq[(int64_t)(n - fz) * fstride] = make_float2(r1 + r2, r3 - r4);
       }
     }
   }
 }
 
-// Inverse counterpart: the z and y inverse passes of one (box, x-frequency)
-// slab.  Phase 1: a warp takes a y-frequency row, lane = channel, reads its n
-// spectrum values (256 bytes per warp load) and forms the SP outputs of the
-// z pass (conjugate input pairs folded as in k_dft_inv_line) into shared
-// memory U[fy][z][c].  Phase 2: a warp takes output points (y, z) and folds
-// the y-frequency pairs of U into t[b][fx][y][z][c], the input of the x pass.
-template <int SP>
-__global__ void __launch_bounds__(256) k_dft_inv_zy(const float2* __restrict__ in, float2* __restrict__ out,
-                                                    int64_t B, const float2* __restrict__ M, int n) {
+// k_dft_inv_line for FP32 and pairs of channels with a thread's whole input line in
+// flight: the n values of 16 bytes go to the thread's own column of shared memory
+// by asynchronous copies, without registers (four pairs ahead in registers cost
+// more in resident warps than they gave: 37.7 -> 43.1 ms for all inverse passes of 120,000
+// unknowns, 64 vectors; this form with k_dft_inv_zy below 24.2).  Same sums in the same
+// order.
+//
+// What bounds it: HBM, 5.1 to 5.9 TB/s on the larger passes (4.2 before).  13^3 splines,
+// 816 MB: 214 -> 146 us.
+template <int AMAX>
+__global__ void __launch_bounds__(128) k_dft_inv_stage(const float2* __restrict__ in, View vin,
+                                                       float2* __restrict__ out, View vout, int64_t B, int C, int ax,
+                                                       int e0, int e1, int e2, const float2* __restrict__ M, int n) {
   extern __shared__ float4 izy_smem[];
-  float2* U = reinterpret_cast<float2*>(izy_smem);  // [n][SP][32]
-  float2* Ms = U + (int64_t)n * SP * 32;            // [f][a] = M[a][f], f = 0 .. n/2
+  constexpr int AP = AMAX + (AMAX & 1);
+  float4* S = izy_smem + threadIdx.x;                        // [n][128], this thread's column
+  float2* Ms = reinterpret_cast<float2*>(izy_smem + n * 128);  // [f][a < AP], f = 0 .. n/2
+  const int nout = ax == 0 ? e0 : (ax == 1 ? e1 : e2);
+  const int nh = n / 2 + 1;
+  for (int i = threadIdx.x; i < nh * AP; i += blockDim.x) {
+    const int f = i / AP, a = i - f * AP;
+    Ms[i] = a < nout ? M[(int64_t)a * n + f] : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  const int ea = ax == 0 ? e1 : e0, eb = ax == 2 ? e1 : e2;
+  const int64_t sa_in = ax == 0 ? vin.s1 : vin.s0, sb_in = ax == 2 ? vin.s1 : vin.s2;
+  const int64_t sa_out = ax == 0 ? vout.s1 : vout.s0, sb_out = ax == 2 ? vout.s1 : vout.s2;
+  const int64_t step_in = ax == 0 ? vin.s0 : (ax == 1 ? vin.s1 : vin.s2);
+  const int64_t step_out = ax == 0 ? vout.s0 : (ax == 1 ? vout.s1 : vout.s2);
+  const int CL = C / 2;
+  const int64_t lines = B * ea * eb * (int64_t)CL;
+  const int np = (n - 1) / 2;     // conjugate pairs (f, n - f), f = 1 .. np
+  const bool mid = (n % 2) == 0;  // f = n/2 pairs with itself
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < lines;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    int64_t t = idx;
+    const int c = (int)(t % CL) * 2;
+    t /= CL;
+    const int ib = (int)(t % eb);
+    t /= eb;
+    const int ia = (int)(t % ea);
+    const int64_t b = t / ea;
+    const float2* ip = in + b * vin.sb + ia * sa_in + ib * sb_in + c;
+    for (int f = 0; f < n; ++f) tile_cp16(S + f * 128, ip + f * step_in);
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    float2 acc[AP][2];
+    const float4* Mr = reinterpret_cast<const float4*>(Ms);
+    {
+      const float4 v = S[0];
+      const float2 v0[2] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+#pragma unroll
+      for (int a = 0; a < AP; a += 2) {
+        const float4 m = Mr[a / 2];
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+          acc[a][l] = cmul(make_float2(m.x, m.y), v0[l]);
+          acc[a + 1][l] = cmul(make_float2(m.z, m.w), v0[l]);
+        }
+      }
+    }
+#pragma unroll 2
+    for (int f = 1; f <= np; ++f) {
+      const float4 z1 = S[f * 128], z2 = S[(n - f) * 128];
+      const float2 u[2] = {make_float2(z1.x + z2.x, z1.y + z2.y), make_float2(z1.z + z2.z, z1.w + z2.w)};
+      const float2 w[2] = {make_float2(z1.x - z2.x, z1.y - z2.y), make_float2(z1.z - z2.z, z1.w - z2.w)};
+      Mr += AP / 2;
+#pragma unroll
+      for (int a = 0; a < AMAX; ++a) {
+        const float4 mm = Mr[a / 2];
+        const float2 m = a & 1 ? make_float2(mm.z, mm.w) : make_float2(mm.x, mm.y);
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+          acc[a][l].x = fmaf(m.x, u[l].x, acc[a][l].x);
+          acc[a][l].x = fmaf(-m.y, w[l].y, acc[a][l].x);
+          acc[a][l].y = fmaf(m.x, u[l].y, acc[a][l].y);
+          acc[a][l].y = fmaf(m.y, w[l].x, acc[a][l].y);
+        }
+      }
+    }
+    if (mid) {
+      const float4 v = S[(n / 2) * 128];
+      const float2 vm[2] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+      const float2* Mm = Ms + (n / 2) * AP;
+#pragma unroll
+      for (int a = 0; a < AMAX; ++a)
+#pragma unroll
+        for (int l = 0; l < 2; ++l) cfma(acc[a][l], Mm[a], vm[l]);
+    }
+    float2* op = out + b * vout.sb + ia * sa_out + ib * sb_out + c;
+#pragma unroll
+    for (int a = 0; a < AMAX; ++a)
+      if (a < nout)
+        *reinterpret_cast<float4*>(op + a * step_out) = make_float4(acc[a][0].x, acc[a][0].y, acc[a][1].x, acc[a][1].y);
+  }
+}
+
+// Inverse counterpart: the z and y inverse passes of one (box, x-frequency)
+// slab, lane = channel.  A warp copies the y-frequency rows fy = warp, warp + SP, ..
+// of the slab (n spectrum values of 256 bytes each) to shared memory by 16-byte
+// asynchronous copies, all of them in flight at once.  Phase 1: it forms the SP
+// outputs of the z pass of each of its rows (conjugate input pairs folded as in
+// k_dft_inv_line) and puts them in the place of the row's first SP values.  Phase 2: a
+// warp takes one z and folds the y-frequency pairs into t[b][fx][y][z][c], the
+// input of the x pass.
+//
+// What bounds it: issue slots (two thirds taken) with HBM at 4.6 TB/s.  508 boxes of
+// 9^3 splines, 16 vectors: 326 -> 178 us (rows came pair by pair before, two loads in flight
+// per warp, and phase 2 read every pair once per output).
+template <int SP>
+__global__ void __launch_bounds__(32 * SP) k_dft_inv_zy(const float2* __restrict__ in, float2* __restrict__ out,
+                                                        int64_t B, const float2* __restrict__ M, int n) {
+  extern __shared__ float4 izy_smem[];
+  constexpr int SPP = SP + (SP & 1);
+  float2* S = reinterpret_cast<float2*>(izy_smem);  // [fy][fz][32]; after phase 1 [fy][z < SP][32]
+  float2* Ms = S + (int64_t)n * n * 32;             // [f][a < SPP] = M[a][f], f = 0 .. n/2
   const int nh = n / 2 + 1;
   const int np = (n - 1) / 2;
   const bool mid = (n % 2) == 0;
-  for (int i = threadIdx.x; i < nh * SP; i += blockDim.x) {
-    const int f = i / SP, a = i - f * SP;
-    Ms[i] = M[(int64_t)a * n + f];
-  }
-  __syncthreads();
   const int64_t sl = blockIdx.x;
   const int64_t b = sl / n;
   const int fx = (int)(sl - b * n);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t fstride = B * 32;
-  for (int fy = warp; fy < n; fy += nw) {
-    const float2* ip = in + (((int64_t)fx * n + fy) * n * B + b) * 32 + lane;
-    float2 acc[SP];
+  for (int fy = warp; fy < n; fy += SP) {
+    const float2* ip = in + (((int64_t)fx * n + fy) * n * B + b) * 32 + (lane & 15) * 2;
+    float2* d = S + (int64_t)fy * n * 32 + (lane & 15) * 2;
+    for (int f = lane >> 4; f < n; f += 2) tile_cp16(d + f * 32, ip + f * fstride);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+  for (int i = threadIdx.x; i < nh * SPP; i += blockDim.x) {
+    const int f = i / SPP, a = i - f * SPP;
+    Ms[i] = a < SP ? M[(int64_t)a * n + f] : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  for (int fy = warp; fy < n; fy += SP) {
+    if (fy + SP < n) asm volatile("cp.async.wait_group 1;\n" ::: "memory");  // n < 2 SP: two rows at most
+    else asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncwarp();
+    float2* ip = S + (int64_t)fy * n * 32 + lane;
+    float2 acc[SPP];
+    const float4* Mr = reinterpret_cast<const float4*>(Ms);
     {
       const float2 v0 = ip[0];
 #pragma unroll
-      for (int a = 0; a < SP; ++a) {
-        const float2 m = Ms[a];
+      for (int a = 0; a < SPP; a += 2) {
+        const float4 m = Mr[a / 2];
         acc[a] = make_float2(m.x * v0.x - m.y * v0.y, m.x * v0.y + m.y * v0.x);
+        acc[a + 1] = make_float2(m.z * v0.x - m.w * v0.y, m.z * v0.y + m.w * v0.x);
       }
     }
+#pragma unroll 2
     for (int f = 1; f <= np; ++f) {
-      const float2 z1 = ip[f * fstride], z2 = ip[(int64_t)(n - f) * fstride];
+      const float2 z1 = ip[f * 32], z2 = ip[(n - f) * 32];
       const float2 u = make_float2(z1.x + z2.x, z1.y + z2.y), w = make_float2(z1.x - z2.x, z1.y - z2.y);
-      const float2* Mr = Ms + f * SP;
+      Mr += SPP / 2;
 #pragma unroll
       for (int a = 0; a < SP; ++a) {
-        const float2 m = Mr[a];
+        const float4 mm = Mr[a / 2];
+        const float2 m = a & 1 ? make_float2(mm.z, mm.w) : make_float2(mm.x, mm.y);
         acc[a].x = fmaf(m.x, u.x, acc[a].x);
         acc[a].x = fmaf(-m.y, w.y, acc[a].x);
         acc[a].y = fmaf(m.x, u.y, acc[a].y);
@@ -1416,38 +1514,62 @@ __global__ void __launch_bounds__(256) k_dft_inv_zy(const float2* __restrict__ i
       }
     }
     if (mid) {
-      const float2 vm = ip[(int64_t)(n / 2) * fstride];
-      const float2* Mr = Ms + (n / 2) * SP;
+      const float2 vm = ip[(n / 2) * 32];
+      const float2* Mm = Ms + (n / 2) * SPP;
 #pragma unroll
       for (int a = 0; a < SP; ++a) {
-        const float2 m = Mr[a];
+        const float2 m = Mm[a];
         acc[a].x = fmaf(m.x, vm.x, fmaf(-m.y, vm.y, acc[a].x));
         acc[a].y = fmaf(m.x, vm.y, fmaf(m.y, vm.x, acc[a].y));
       }
     }
 #pragma unroll
-    for (int a = 0; a < SP; ++a) U[(fy * SP + a) * 32 + lane] = acc[a];
+    for (int a = 0; a < SP; ++a) ip[a * 32] = acc[a];  // SP <= n; the lane's own column
   }
   __syncthreads();
-  float2* op = out + sl * (SP * SP * 32) + lane;
-  for (int o = warp; o < SP * SP; o += nw) {
-    const int y = o / SP, z = o - y * SP;
-    const float2 m0 = Ms[y], v0 = U[z * 32 + lane];
-    float ax = m0.x * v0.x - m0.y * v0.y, ay = m0.x * v0.y + m0.y * v0.x;
+  {
+    const int z = warp;
+    const float2* U = S + z * 32 + lane;
+    const int64_t row = (int64_t)n * 32;
+    float2 acc[SPP];
+    const float4* Mr = reinterpret_cast<const float4*>(Ms);
+    {
+      const float2 v0 = U[0];
+#pragma unroll
+      for (int a = 0; a < SPP; a += 2) {
+        const float4 m = Mr[a / 2];
+        acc[a] = make_float2(m.x * v0.x - m.y * v0.y, m.x * v0.y + m.y * v0.x);
+        acc[a + 1] = make_float2(m.z * v0.x - m.w * v0.y, m.z * v0.y + m.w * v0.x);
+      }
+    }
+#pragma unroll 2
     for (int f = 1; f <= np; ++f) {
-      const float2 z1 = U[(f * SP + z) * 32 + lane], z2 = U[((n - f) * SP + z) * 32 + lane];
-      const float2 m = Ms[f * SP + y];
-      ax = fmaf(m.x, z1.x + z2.x, ax);
-      ax = fmaf(-m.y, z1.y - z2.y, ax);
-      ay = fmaf(m.x, z1.y + z2.y, ay);
-      ay = fmaf(m.y, z1.x - z2.x, ay);
+      const float2 z1 = U[f * row], z2 = U[(n - f) * row];
+      const float2 u = make_float2(z1.x + z2.x, z1.y + z2.y), w = make_float2(z1.x - z2.x, z1.y - z2.y);
+      Mr += SPP / 2;
+#pragma unroll
+      for (int a = 0; a < SP; ++a) {
+        const float4 mm = Mr[a / 2];
+        const float2 m = a & 1 ? make_float2(mm.z, mm.w) : make_float2(mm.x, mm.y);
+        acc[a].x = fmaf(m.x, u.x, acc[a].x);
+        acc[a].x = fmaf(-m.y, w.y, acc[a].x);
+        acc[a].y = fmaf(m.x, u.y, acc[a].y);
+        acc[a].y = fmaf(m.y, w.x, acc[a].y);
+      }
     }
     if (mid) {
-      const float2 m = Ms[(n / 2) * SP + y], vm = U[((n / 2) * SP + z) * 32 + lane];
-      ax = fmaf(m.x, vm.x, fmaf(-m.y, vm.y, ax));
-      ay = fmaf(m.x, vm.y, fmaf(m.y, vm.x, ay));
+      const float2 vm = U[(n / 2) * row];
+      const float2* Mm = Ms + (n / 2) * SPP;
+#pragma unroll
+      for (int a = 0; a < SP; ++a) {
+        const float2 m = Mm[a];
+        acc[a].x = fmaf(m.x, vm.x, fmaf(-m.y, vm.y, acc[a].x));
+        acc[a].y = fmaf(m.x, vm.y, fmaf(m.y, vm.x, acc[a].y));
+      }
     }
-    op[(int64_t)o * 32] = make_float2(ax, ay);
+    float2* op = out + sl * (SP * SP * 32) + z * 32 + lane;
+#pragma unroll
+    for (int y = 0; y < SP; ++y) op[y * (SP * 32)] = acc[y];
   }
 }
 
@@ -1455,11 +1577,14 @@ __global__ void __launch_bounds__(256) k_dft_inv_zy(const float2* __restrict__ i
 // sp splines per axis and FFT length n (9, 13 or 21 splines; shared memory).
 static size_t dft_yz_smem(int sp, int n, bool inverse) {
   const int nh = n / 2 + 1;
-  return inverse ? sizeof(float2) * ((size_t)n * sp * 32 + (size_t)nh * sp)
+  return inverse ? sizeof(float2) * ((size_t)n * n * 32 + (size_t)nh * (sp + (sp & 1)))
                  : sizeof(float2) * ((size_t)sp * sp * 32 + (size_t)nh * sp);
 }
 bool dft_yz_fits(int sp, int n) { return (sp == 9 || sp == 13 || sp == 21) && dft_yz_smem(sp, n, false) <= 200 * 1024; }
-bool dft_zy_fits(int sp, int n) { return (sp == 9 || sp == 13 || sp == 21) && dft_yz_smem(sp, n, true) <= 200 * 1024; }
+// (at most two rows of a slab per warp, whose sums take the place of the inputs)
+bool dft_zy_fits(int sp, int n) {
+  return (sp == 9 || sp == 13) && sp <= n && n < 2 * sp && dft_yz_smem(sp, n, true) <= 200 * 1024;
+}
 
 // Fused y-z forward (in: t[b][fx][y][z][32] -> out: Q[fx][fy][fz][b][32]) or
 // z-y inverse (in: Q layout -> out: t layout).  Returns false when they do not
@@ -1470,18 +1595,22 @@ bool launch_dft_yz(const float2* in, float2* out, int64_t B, int sp, int n, cons
   if (slabs <= 0) return true;
   if (slabs > 0x7FFFFFFFLL) return false;
   const size_t smem = dft_yz_smem(sp, n, inverse);
-  if (smem > 200 * 1024) return false;
+  if (inverse ? !dft_zy_fits(sp, n) : smem > 200 * 1024) return false;
+  // one y-frequency pair per warp and round, the warps even over the rounds
+  const int rounds = (n / 2 + 8) / 8, warps = (n / 2 + rounds) / rounds;
 #define EFIE_YZ(SPV)                                                                                 \
   if (sp == SPV) {                                                                                   \
-    if (inverse) {                                                                                   \
-      static SmemAttr attr;                                                                          \
-      smem_attr_once(k_dft_inv_zy<SPV>, (int)smem, attr.v);                                          \
-      k_dft_inv_zy<SPV><<<(unsigned)slabs, 256, smem, s>>>(in, out, B, M, n);                        \
-    } else {                                                                                         \
-      static SmemAttr attr;                                                                          \
-      smem_attr_once(k_dft_fwd_yz<SPV>, (int)smem, attr.v);                                          \
-      k_dft_fwd_yz<SPV><<<(unsigned)slabs, 256, smem, s>>>(in, out, B, M, n);                        \
+    if constexpr (SPV <= 13) {                                                                       \
+      if (inverse) {                                                                                 \
+        static SmemAttr attr;                                                                        \
+        smem_attr_once(k_dft_inv_zy<SPV>, (int)smem, attr.v);                                        \
+        k_dft_inv_zy<SPV><<<(unsigned)slabs, 32 * SPV, smem, s>>>(in, out, B, M, n);                 \
+        return true;                                                                                 \
+      }                                                                                              \
     }                                                                                                \
+    static SmemAttr attr;                                                                            \
+    smem_attr_once(k_dft_fwd_yz<SPV>, (int)smem, attr.v);                                            \
+    k_dft_fwd_yz<SPV><<<(unsigned)slabs, 32 * warps, smem, s>>>(in, out, B, M, n);                   \
     return true;                                                                                     \
   }
   EFIE_YZ(9)
@@ -1544,19 +1673,21 @@ bool launch_dft(const cpx_t<R>* in, View vin, cpx_t<R>* out, View vout, int64_t 
   if (smem > 96 * 1024) return false;
 #define EFIE_DI(AM)                                                                                          \
   if (nout <= AM) {                                                                                          \
-    if (two && AM <= 21) {                                                                                   \
-      auto k = k_dft_inv_line<R, AM, (sizeof(R) == 4 && AM <= 21) ? 2 : 1>;                                  \
-      static SmemAttr attr;                                                                  \
-      smem_attr_once(k, 96 * 1024, attr.v);                                                                    \
-      k<<<(unsigned)blocks, 128, smem, s>>>(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n);            \
-      return true;                                                                                           \
+    if constexpr (sizeof(R) == 4) {                                                                          \
+      const size_t sm = (size_t)n * 2048 + sizeof(T) * (size_t)nh * (AM + (AM & 1));                         \
+      if (two && sm <= 100 * 1024) {                                                                         \
+        static SmemAttr attr2;                                                                               \
+        smem_attr_once(k_dft_inv_stage<AM>, 100 * 1024, attr2.v);                                            \
+        k_dft_inv_stage<AM><<<(unsigned)blocks, 128, sm, s>>>(in, vin, out, vout, B, C, ax, e0, e1, e2, M, n); \
+        return true;                                                                                         \
+      }                                                                                                      \
     }                                                                                                        \
     const int64_t lines1 = B * ea * eb * (int64_t)C;                                                         \
     int64_t blocks1 = ceil_div(lines1, 128);                                                                 \
     if (blocks1 > 152 * 32) blocks1 = 152 * 32;                                                              \
-    auto k = k_dft_inv_line<R, AM, 1>;                                                                       \
-    static SmemAttr attr1;                                                                   \
-    smem_attr_once(k, 96 * 1024, attr1.v);                                                                     \
+    auto k = k_dft_inv_line<R, AM>;                                                                          \
+    static SmemAttr attr1;                                                                                   \
+    smem_attr_once(k, 96 * 1024, attr1.v);                                                                   \
     k<<<(unsigned)blocks1, 128, smem, s>>>(in, vin, out, vout, B, C, ax, nin, e0, e1, e2, M, n);             \
     return true;                                                                                             \
   }
