@@ -2429,83 +2429,19 @@ __global__ void __launch_bounds__(128) k_mac_top32(const float2* __restrict__ Qh
   }
 }
 
-// Interaction-list levels, FP32: the kernel values of one frequency are at most
-// O (<= 316 on these levels) complex numbers; every block stages the rows of its
-// fpb frequencies in shared memory, so the per-pair kernel lookups hit shared
-// memory and only the spectra come from L1/L2.
-template <int XR, int CR>
-__global__ void __launch_bounds__(128) k_mac_il32(const float2* __restrict__ Qh, float2* __restrict__ Rh,
-                                                  const float2* __restrict__ Kh, int64_t B, int C, int64_t O,
-                                                  int64_t nf, const int64_t* __restrict__ tgt_ptr,
-                                                  const int32_t* __restrict__ tgt,
-                                                  const int64_t* __restrict__ src_ptr,
-                                                  const int32_t* __restrict__ src,
-                                                  const int64_t* __restrict__ kidx_off,
-                                                  const int32_t* __restrict__ kidx, int fpb, int64_t f0) {
-  extern __shared__ __align__(16) unsigned char mac_smem[];
-  float2* Kr = reinterpret_cast<float2*>(mac_smem);   // [fpb][O]
-  const int tile = blockIdx.x;
-  const int64_t fb = f0 + (int64_t)blockIdx.y * fpb;
-  for (int e = threadIdx.x; e < fpb * O; e += blockDim.x) {
-    const int fl = e / (int)O;
-    const int64_t f = fb + fl;
-    Kr[e] = f < nf ? __ldg(Kh + f * O + (e - fl * O)) : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  const int ncg = C / CR;
-  const int fl = threadIdx.x / ncg, cg = threadIdx.x - fl * ncg;
-  const int64_t f = fb + fl;
-  if (fl >= fpb || f >= nf) return;
-  const int64_t t0 = tgt_ptr[tile], nt = tgt_ptr[tile + 1] - t0;
-  const int64_t s0 = src_ptr[tile], ns = src_ptr[tile + 1] - s0;
-  const int32_t* kb = kidx + kidx_off[tile];
-  const float2* Qf = Qh + f * B * C + cg * CR;
-  const float2* Kf = Kr + fl * O;
-  float2 acc[XR][CR];
-#pragma unroll
-  for (int a = 0; a < XR; ++a)
-#pragma unroll
-    for (int c = 0; c < CR; ++c) acc[a][c] = make_float2(0.f, 0.f);
-  for (int64_t j = 0; j < ns; ++j) {
-    const int32_t y = __ldg(src + s0 + j);
-    float2 q[CR];
-#pragma unroll
-    for (int c2 = 0; c2 < CR; c2 += 2) {
-      const float4 qa = __ldg(reinterpret_cast<const float4*>(Qf + (int64_t)y * C + c2));
-      q[c2] = make_float2(qa.x, qa.y);
-      q[c2 + 1] = make_float2(qa.z, qa.w);
-    }
-    const int4 ia = __ldg(reinterpret_cast<const int4*>(kb + j * XR));
-    const int4 ib = __ldg(reinterpret_cast<const int4*>(kb + j * XR + 4));
-    const int ids[8] = {ia.x, ia.y, ia.z, ia.w, ib.x, ib.y, ib.z, ib.w};
-#pragma unroll
-    for (int a = 0; a < XR; ++a) {
-      if (ids[a] < 0) continue;
-      const float2 kv = Kf[ids[a]];
-#pragma unroll
-      for (int c = 0; c < CR; ++c) cfma(acc[a][c], kv, q[c]);
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < XR; ++a) {
-    if (a >= nt) break;
-    float2* out = Rh + f * B * C + (int64_t)tgt[t0 + a] * C + cg * CR;
-#pragma unroll
-    for (int c2 = 0; c2 < CR; c2 += 2)
-      *reinterpret_cast<float4*>(out + c2) =
-          make_float4(acc[a][c2].x, acc[a][c2].y, acc[a][c2 + 1].x, acc[a][c2 + 1].y);
-  }
-}
-
-// Translation from the interaction lists: a thread owns 16 bytes of one
-// (frequency, target) and runs down the target's list, four pairs in flight.  The
+// Translation from the interaction lists: a thread owns NU units of 16 bytes of one
+// (frequency, target) and runs down the target's list, four pairs in flight; NU = 2
+// takes the list entry and the kernel value once for twice the products.  The
 // register tiles of k_mac_tiled visit every (source, target) slot of a tile, pairs or
 // not (FP64 multiply-adds of excluded slots cost as much as the others), and leave
-// most of the chip idle on few tiles and channels.  Sources ascend in both, so
-// the sums are the same bit for bit.  ms: 1,920 unknowns, FP64, one vector 0.076 ->
-// 0.045; 6,750, FP32, one vector 0.065 -> 0.032; 48,000, FP32, one vector, leaf level
-// 0.33 -> 0.16; 48,000, FP64, 8 vectors, top level 31.1 -> 27.8.
-template <typename R>
+// most of the chip idle on few tiles and channels; a kernel with the kernel rows of
+// eight frequencies in shared memory and 8 targets per thread waited for its dependent
+// loads.  Sources ascend in all of them, so the sums are the same bit for bit.  What
+// bounds it: L1 requests.  ms: 1,920 unknowns, FP64, one vector 0.076 -> 0.045; 6,750,
+// FP32, one vector 0.065 -> 0.032; 48,000, FP32, leaf level, one vector 0.33 -> 0.16, 4
+// vectors 0.81 -> 0.36, 8 vectors 0.76 -> 0.59; 48,000, FP64, 8 vectors, top level
+// 31.1 -> 27.8.
+template <typename R, int NU>
 __global__ void __launch_bounds__(128) k_mac_list(const typename U16<R>::T* __restrict__ Qh,
                                                   typename U16<R>::T* __restrict__ Rh,
                                                   const cpx_t<R>* __restrict__ Kh, int64_t B, int U, int64_t O,
@@ -2514,34 +2450,50 @@ __global__ void __launch_bounds__(128) k_mac_list(const typename U16<R>::T* __re
                                                   const int32_t* __restrict__ il_off, int64_t f0) {
   using T = typename U16<R>::T;
   const int64_t t = (int64_t)blockIdx.x * 128 + threadIdx.x;
-  const int64_t x = t / U, f = f0 + blockIdx.y;
-  const int u = (int)(t - x * U);
+  const int US = U / NU;
+  const int64_t x = t / US, f = f0 + blockIdx.y;
+  const int u = (int)(t - x * US);
   if (x >= B) return;
   const T* Qf = Qh + f * B * U + u;
   const cpx_t<R>* Kf = Kh + f * O;
-  T acc = U16<R>::zero();
+  T acc[NU];
+#pragma unroll
+  for (int v = 0; v < NU; ++v) acc[v] = U16<R>::zero();
   const int64_t e1 = il_ptr[x + 1];
   int64_t e = il_ptr[x];
-  const auto mac = [&](const cpx_t<R>& k, const T& q) {
-    cpx_t<R> a = mk<R>(acc.x, acc.y);
+  const auto mac = [&](T& s, const cpx_t<R>& k, const T& q) {
+    cpx_t<R> a = mk<R>(s.x, s.y);
     cfma(a, k, mk<R>(q.x, q.y));
-    acc.x = a.x, acc.y = a.y;
+    s.x = a.x, s.y = a.y;
     if constexpr (sizeof(R) == 4) {
-      a = mk<R>(acc.z, acc.w);
+      a = mk<R>(s.z, s.w);
       cfma(a, k, mk<R>(q.z, q.w));
-      acc.z = a.x, acc.w = a.y;
+      s.z = a.x, s.w = a.y;
     }
   };
   for (; e + 4 <= e1; e += 4) {
     cpx_t<R> k[4];
-    T q[4];
+    T q[4][NU];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) k[i] = Kf[__ldg(il_off + e + i)], q[i] = __ldg(Qf + (int64_t)__ldg(il_src + e + i) * U);
+    for (int i = 0; i < 4; ++i) {
+      k[i] = Kf[__ldg(il_off + e + i)];
+      const T* qp = Qf + (int64_t)__ldg(il_src + e + i) * U;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) mac(k[i], q[i]);
+      for (int v = 0; v < NU; ++v) q[i][v] = __ldg(qp + v * US);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int v = 0; v < NU; ++v) mac(acc[v], k[i], q[i][v]);
   }
-  for (; e < e1; ++e) mac(Kf[__ldg(il_off + e)], __ldg(Qf + (int64_t)__ldg(il_src + e) * U));
-  Rh[(f * B + x) * U + u] = acc;
+  for (; e < e1; ++e) {
+    const cpx_t<R> k = Kf[__ldg(il_off + e)];
+    const T* qp = Qf + (int64_t)__ldg(il_src + e) * U;
+#pragma unroll
+    for (int v = 0; v < NU; ++v) mac(acc[v], k, __ldg(qp + v * US));
+  }
+#pragma unroll
+  for (int v = 0; v < NU; ++v) Rh[(f * B + x) * U + u + v * US] = acc[v];
 }
 
 template <typename R>
@@ -2566,53 +2518,49 @@ void launch_mac(const cpx_t<R>* Qh, cpx_t<R>* Rh, const cpx_t<R>* Kh, int64_t B,
     }
     return;
   }
-  if (!force_reg && sizeof(R) == 4 && (C % 2) == 0 && C >= 16 && max_tile_targets <= 8 && O <= 2048) {
-    // interaction-list tiles (<= 8 targets): kernel rows of fpb frequencies in
-    // shared memory; CRI channels per thread (2: fewer registers, more warps
-    // in flight for this latency-bound loop)
-    constexpr int CRI = 2;
-    const int ncg = C / CRI;
-    int fpb = 128 / ncg;
-    if (fpb < 1) fpb = 1;
-    while (fpb > 1 && (size_t)fpb * O * sizeof(float2) > 64 * 1024) fpb >>= 1;
-    const size_t smem = (size_t)fpb * O * sizeof(float2);
-    static SmemAttr attr;
-    smem_attr_once(k_mac_il32<8, CRI>, 64 * 1024, attr.v);
+  // From the lists: in FP64 always; in FP32 on interaction-list tiles (at most 8
+  // targets), on top levels of at most 64 boxes, and otherwise for 12 channels and
+  // more that are no multiple of 8 (128 boxes, 21^3 frequencies, 12, 20 and 28
+  // channels: 1.02, 1.72 and 2.21 ms in register tiles, 0.98, 1.47 and 1.89 from the
+  // lists).  Wide tiles of 4 channels reuse each kernel value for more products (0.51 ms
+  // against 0.57), and those of 8, 16 and 24 take 8 channels per thread (0.83, 1.27
+  // and 1.78 ms with 4; 0.68, 1.15 and 1.51 with 8; 0.76, 1.14 and 1.64 from the lists).
+  const bool wide = max_tile_targets > 8 && !(ntiles == 1 && max_tile_targets <= 64);
+  const bool cr8 = sizeof(R) == 4 && C % 8 == 0 && !force_reg;
+  if (!force_reg && (sizeof(R) == 8 || !wide || (C >= 12 && !cr8))) {
+    const int U = C * (int)sizeof(cpx_t<R>) / 16;
+    const auto run = [&](auto k, int nu) {
+      const unsigned gx = (unsigned)ceil_div(B * (U / nu), 128);
+      for (int64_t f0 = 0; f0 < nf; f0 += 65535)
+        k<<<dim3(gx, (unsigned)std::min<int64_t>(65535, nf - f0)), 128, 0, s>>>(
+            reinterpret_cast<const typename U16<R>::T*>(Qh), reinterpret_cast<typename U16<R>::T*>(Rh), Kh, B, U, O,
+            il_ptr, il_src, il_off, f0);
+    };
+    // two units per thread where there are enough (FP32; 8 channels: 0.171 ms with
+    // one on the leaf level of 21,870 unknowns, 0.181 with two; 16: 0.284 and 0.255)
+    if constexpr (sizeof(R) == 4) {
+      if (C >= 12 && U % 2 == 0) return run(k_mac_list<R, 2>, 2);
+    }
+    return run(k_mac_list<R, 1>, 1);
+  }
+  constexpr int XR = 8;
+  const auto run = [&](auto k, int cr) {
+    const int ncg = C / cr;
+    const int ntx = (max_tile_targets + XR - 1) / XR;
+    const int per_f = ntx * ncg;
+    const int fpb = per_f >= 128 ? 1 : 128 / per_f;
+    const int threads = fpb * per_f;
     const int64_t fchunk = (int64_t)65535 * fpb;
     for (int64_t f0 = 0; f0 < nf; f0 += fchunk) {
       int64_t nfc = std::min<int64_t>(fchunk, nf - f0);
       dim3 grid((unsigned)ntiles, (unsigned)ceil_div(nfc, fpb));
-      k_mac_il32<8, CRI><<<grid, fpb * ncg, smem, s>>>((const float2*)Qh, (float2*)Rh, (const float2*)Kh, B, C, O,
-                                                       nf, tgt_ptr, tgt, src_ptr, src, kidx_off, kidx, fpb, f0);
+      k<<<grid, threads, 0, s>>>(Qh, Rh, Kh, B, C, O, nf, tgt_ptr, tgt, src_ptr, src, kidx_off, kidx, fpb, ntx, f0);
     }
-    return;
+  };
+  if constexpr (sizeof(R) == 4) {
+    if (cr8) return run(k_mac_tiled<R, XR, 8>, 8);
   }
-  // In FP64 always.  In FP32 on interaction-list tiles (at most 8 targets), and on
-  // top levels of at most 64 boxes; wider tiles of one list reuse each kernel value
-  // for more products (128 boxes, 21^3 frequencies, 4 channels: 0.51 ms in register
-  // tiles, 0.57 from the lists).
-  if (!force_reg && (sizeof(R) == 8 || max_tile_targets <= 8 || (ntiles == 1 && max_tile_targets <= 64))) {
-    const int U = C * (int)sizeof(cpx_t<R>) / 16;
-    const unsigned gx = (unsigned)ceil_div(B * U, 128);
-    for (int64_t f0 = 0; f0 < nf; f0 += 65535)
-      k_mac_list<R><<<dim3(gx, (unsigned)std::min<int64_t>(65535, nf - f0)), 128, 0, s>>>(
-          reinterpret_cast<const typename U16<R>::T*>(Qh), reinterpret_cast<typename U16<R>::T*>(Rh), Kh, B, U, O, il_ptr,
-          il_src, il_off, f0);
-    return;
-  }
-  constexpr int XR = 8, CR = 4;
-  const int ncg = C / CR;
-  const int ntx = (max_tile_targets + XR - 1) / XR;
-  const int per_f = ntx * ncg;
-  int fpb = per_f >= 128 ? 1 : 128 / per_f;
-  const int threads = fpb * per_f;
-  const int64_t fchunk = (int64_t)65535 * fpb;
-  for (int64_t f0 = 0; f0 < nf; f0 += fchunk) {
-    int64_t nfc = std::min<int64_t>(fchunk, nf - f0);
-    dim3 grid((unsigned)ntiles, (unsigned)ceil_div(nfc, fpb));
-    k_mac_tiled<R, XR, CR><<<grid, threads, 0, s>>>(Qh, Rh, Kh, B, C, O, nf, tgt_ptr, tgt, src_ptr, src, kidx_off,
-                                                    kidx, fpb, ntx, f0);
-  }
+  run(k_mac_tiled<R, XR, 4>, 4);
 }
 
 // ---------------------------------------------------------------- kernel samples

@@ -1,8 +1,9 @@
 """The FP64 translation's forms at the edges of their tiles: leaf boxes that are no
 multiple of 16, unions that are no multiple of 8, and 4, 12, 20 and 32
 channels (1, 3, 5 and 8 vectors), the tensor-core form against the oracle and against the
-register tiles; the mixed form's list translation (1 and 3 vectors) against its
-register tiles, whose sums it repeats bit for bit."""
+register tiles; the mixed form's list translation (one and two units per thread) and
+its wide tiles of 8 channels per thread against the register tiles, whose sums they
+repeat bit for bit."""
 import numpy as np
 import pytest
 
@@ -51,13 +52,19 @@ def test_fp64_forms(case):
         h.close()
 
 
-def test_mixed_lists_repeat_the_tiles(case):
+@pytest.mark.parametrize("wide", [False, True])
+def test_mixed_lists_repeat_the_tiles(case, wide):
     import paper_2606_13482_gb300 as G
     args, X, _ = case
+    if wide:   # more than 64 boxes on the top level
+        V, T = E.icosphere(28, 2.0)
+        args = (V, T) + args[2:]
+        X = E.complex_gaussian((7, 3 * len(T) // 2), 82)
+        assert G.plan(*args)[1][-1]["n_boxes"] > 64 and G.plan(*args)[1][0]["n_boxes"] > 64
     h = G.EFIE(*args, precision=G.EFIE_MIXED)
     try:
-        for n in (1, 3):
-            assert np.array_equal(_products(h, X, 0, n), _products(h, X, 1, n))
+        for n in (1, 2, 3, 4, 5, 6, 7):
+            assert np.array_equal(_products(h, X, 0, n), _products(h, X, 1, n)), n
     finally:
         h.close()
 
