@@ -403,7 +403,8 @@ int efie_autotune_set(efie_handle *h, int rhs_chunk, int mac_variant, int near_v
  * right-hand sides (32 channels) and 9, 13 or 21 splines per axis, the
  * forward y and z passes run fused on (box, x-frequency) slabs in shared
  * memory, so the intermediate of the second pass never goes to device
- * memory; 2: the inverse z and y passes fused the same way as well; 3
+ * memory; 2: the inverse z and y passes of 9 and 13 splines fused the same
+ * way as well; 3
  * (default): forward and inverse fused on levels of 9 splines per axis only,
  * line passes on the others.  All give the same operator up to rounding.
  * efie_autotune times all four (after choosing the other knobs) for mixed

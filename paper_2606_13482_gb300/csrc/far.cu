@@ -1269,7 +1269,7 @@ bool launch_dft_fold(const double2* in, View vin, double2* out, View vout, int64
 // warp store).  The y-pass intermediate never goes to HBM: per box the pass
 // pair reads n SP^2 and writes n^3 values instead of reading and writing
 // n SP^2 + n^2 SP.  What bounds it: issue slots (two thirds taken) with HBM at
-// 4.5 TB/s.  508 boxes of 9^3 splines, 16 vectors: 215 -> 175 us (one matrix read per
+// 4.5 TB/s.  1,016 boxes of 9^3 splines, 16 vectors: 215 -> 175 us (one matrix read per
 // row and a warp of eight idle before).
 template <int SP>
 __global__ void __launch_bounds__(256, SP == 9 ? 3 : 1)
@@ -1351,7 +1351,7 @@ __global__ void __launch_bounds__(256, SP == 9 ? 3 : 1)
 // k_dft_inv_line for FP32 and pairs of channels with a thread's whole input line in
 // flight: the n values of 16 bytes go to the thread's own column of shared memory
 // by asynchronous copies, without registers (four pairs ahead in registers cost
-// more in resident warps than they gave: 37.7 -> 43.1 ms for all inverse passes of 120,000
+// more in resident warps than they gave: 37.7 -> 43.1 ms for all inverse passes of 300,000
 // unknowns, 64 vectors; this form with k_dft_inv_zy below 24.2).  Same sums in the same
 // order.
 //
@@ -1453,7 +1453,7 @@ __global__ void __launch_bounds__(128) k_dft_inv_stage(const float2* __restrict_
 // warp takes one z and folds the y-frequency pairs into t[b][fx][y][z][c], the
 // input of the x pass.
 //
-// What bounds it: issue slots (two thirds taken) with HBM at 4.6 TB/s.  508 boxes of
+// What bounds it: issue slots (two thirds taken) with HBM at 4.6 TB/s.  1,016 boxes of
 // 9^3 splines, 16 vectors: 326 -> 178 us (rows came pair by pair before, two loads in flight
 // per warp, and phase 2 read every pair once per output).
 template <int SP>
