@@ -1598,24 +1598,21 @@ bool launch_dft_yz(const float2* in, float2* out, int64_t B, int sp, int n, cons
   if (inverse ? !dft_zy_fits(sp, n) : smem > 200 * 1024) return false;
   // one y-frequency pair per warp and round, the warps even over the rounds
   const int rounds = (n / 2 + 8) / 8, warps = (n / 2 + rounds) / rounds;
-#define EFIE_YZ(SPV)                                                                                 \
-  if (sp == SPV) {                                                                                   \
-    if constexpr (SPV <= 13) {                                                                       \
-      if (inverse) {                                                                                 \
-        static SmemAttr attr;                                                                        \
-        smem_attr_once(k_dft_inv_zy<SPV>, (int)smem, attr.v);                                        \
-        k_dft_inv_zy<SPV><<<(unsigned)slabs, 32 * SPV, smem, s>>>(in, out, B, M, n);                 \
-        return true;                                                                                 \
-      }                                                                                              \
-    }                                                                                                \
-    static SmemAttr attr;                                                                            \
-    smem_attr_once(k_dft_fwd_yz<SPV>, (int)smem, attr.v);                                            \
-    k_dft_fwd_yz<SPV><<<(unsigned)slabs, 32 * warps, smem, s>>>(in, out, B, M, n);                   \
-    return true;                                                                                     \
+#define EFIE_YZ(SPV, KERNEL, WARPS)                                             \
+  if (sp == SPV) {                                                              \
+    static SmemAttr attr;                                                       \
+    smem_attr_once(KERNEL<SPV>, (int)smem, attr.v);                             \
+    KERNEL<SPV><<<(unsigned)slabs, 32 * (WARPS), smem, s>>>(in, out, B, M, n);  \
+    return true;                                                                \
   }
-  EFIE_YZ(9)
-  EFIE_YZ(13)
-  EFIE_YZ(21)
+  if (inverse) {
+    EFIE_YZ(9, k_dft_inv_zy, 9)
+    EFIE_YZ(13, k_dft_inv_zy, 13)
+    return false;
+  }
+  EFIE_YZ(9, k_dft_fwd_yz, warps)
+  EFIE_YZ(13, k_dft_fwd_yz, warps)
+  EFIE_YZ(21, k_dft_fwd_yz, warps)
 #undef EFIE_YZ
   return false;
 }
@@ -1839,8 +1836,9 @@ __global__ void k_gather_build(const R* __restrict__ mr, const int32_t* __restri
 // over the sorted lists).  LR lanes, the right-hand sides rounded up to a power
 // of two, share a point: a warp takes 32 / LR points at a time, the lanes of a
 // point read the same list entry (one broadcast) and consecutive staged values,
-// and own their 4 output components outright -- no atomics, no reductions,
-// each moment entry read once per launch, each output written once.
+// and own their 4 output components outright -- no atomics, each moment entry read
+// once per launch, each output written once.  In FP64, SPL groups of LR lanes share a
+// point's list entry by entry and add their sums by shuffles.
 //
 // What bounds it: the latency of the list entries, and in FP64 the multiply-
 // adds, so lanes without a right-hand side (7 of 8 with LR = 8 and one vector)
@@ -1848,7 +1846,10 @@ __global__ void k_gather_build(const R* __restrict__ mr, const int32_t* __restri
 // few boxes.  Measured: 1,920 unknowns, 32 boxes, FP64, one vector
 // 0.397 -> 0.078 ms; 48,000 unknowns, FP64, 8 vectors 2.75 -> 1.31 (two passes per 32
 // points before); the nonuniform tree with 22 leaves of 41^3 points on its top
-// level, 64 vectors 166 -> 5.8.
+// level, 64 vectors 166 -> 5.8.  FP64 with lists shared by SPL groups (8 to 16 lanes a
+// point; half or twice as many measured slower on small or on large trees), 1, 2, 4 and
+// 8 vectors: 1,920 unknowns in one level 0.188 -> 0.036, 0.182 -> 0.056, 0.165 -> 0.066,
+// 0.175 -> 0.114; 48,000 unknowns 0.398 -> 0.331, 0.528 -> 0.451, 0.816 -> 0.695, 1.28 -> 1.07.
 template <typename R, int LR>
 struct AnterpCfg {
   // values per staged function: rows of 80 bytes (FP32) and 144 (FP64) spread the banks
@@ -1856,7 +1857,7 @@ struct AnterpCfg {
 };
 constexpr int ANTERP_SMEM = 96 * 1024;
 
-template <typename R, int LR>
+template <typename R, int LR, int SPL>
 __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const R* __restrict__ gt,
                                                 const int32_t* __restrict__ gptr_r,
                                                 const int32_t* __restrict__ gptr_t,
@@ -1869,7 +1870,7 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
                                                 const cpx_t<R>* __restrict__ rho, int64_t ldr, int nr,
                                                 cpx_t<R>* __restrict__ q, int sp, int ak, int at, int nsplit) {
   using T = cpx_t<R>;
-  constexpr int XS = AnterpCfg<R, LR>::XS, PW = 32 / LR;
+  constexpr int XS = AnterpCfg<R, LR>::XS, PW = 32 / (LR * SPL);
   extern __shared__ __align__(16) unsigned char anterp_smem[];
   T* xsm = reinterpret_cast<T*>(anterp_smem);  // [ak][XS]
   T* rsm = xsm + (size_t)ak * XS;              // [at][XS]
@@ -1897,7 +1898,7 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
     stage(0);
     __syncthreads();
   }
-  const int r = lane & (LR - 1), ps = lane / LR;
+  const int r = lane & (LR - 1), lp = lane / LR & (SPL - 1), ps = lane / (LR * SPL);
   const int C = 4 * nr;
   const int per_pass = PW * (blockDim.x >> 5);
   // passes part, part + nsplit, ..: points near the surface, where the lists
@@ -1906,8 +1907,8 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
     const int p = pb + PW * warp + ps;
     const bool okp = p < npts;
     T a0 = mk<R>(0, 0), a1 = a0, a2 = a0, a3 = a0;
-    int er = okp ? pr[p] : 0, er1 = okp ? pr[p + 1] : 0;
-    int et = okp ? pq[p] : 0, et1 = okp ? pq[p + 1] : 0;
+    int er = okp ? pr[p] + lp : 0, er1 = okp ? pr[p + 1] : 0;
+    int et = okp ? pq[p] + lp : 0, et1 = okp ? pq[p + 1] : 0;
     for (int c = 0; c < nchunk; ++c) {
       if (nchunk > 1) {
         __syncthreads();
@@ -1936,15 +1937,15 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
       };
       if (nchunk == 1) {
         // every entry belongs to this chunk: four list entries in flight at a time
-        for (; er + 3 < er1; er += 4) {
+        for (; er + 3 * SPL < er1; er += 4 * SPL) {
           R k_[4], x_[4], y_[4], z_[4];
 #pragma unroll
-          for (int t = 0; t < 4; ++t) load4(er + t, k_[t], x_[t], y_[t], z_[t]);
+          for (int t = 0; t < 4; ++t) load4(er + t * SPL, k_[t], x_[t], y_[t], z_[t]);
 #pragma unroll
           for (int t = 0; t < 4; ++t) mac3((int)k_[t], x_[t], y_[t], z_[t]);
         }
       }
-      for (; er < er1; ++er) {
+      for (; er < er1; er += SPL) {
         R ek, m0, m1, m2;
         load4(er, ek, m0, m1, m2);
         if ((int)ek >= kc0 + ak) break;
@@ -1966,22 +1967,30 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
         a3.y = fma(m, v.y, a3.y);
       };
       if (nchunk == 1) {
-        for (; et + 3 < et1; et += 4) {
+        for (; et + 3 * SPL < et1; et += 4 * SPL) {
           R k_[4], m_[4];
 #pragma unroll
-          for (int t = 0; t < 4; ++t) load2(et + t, k_[t], m_[t]);
+          for (int t = 0; t < 4; ++t) load2(et + t * SPL, k_[t], m_[t]);
 #pragma unroll
           for (int t = 0; t < 4; ++t) mac1((int)k_[t], m_[t]);
         }
       }
-      for (; et < et1; ++et) {
+      for (; et < et1; et += SPL) {
         R ek, m;
         load2(et, ek, m);
         if ((int)ek >= tc0 + at) break;
         mac1((int)ek, m);
       }
     }
-    if (okp && r < nr) {
+#pragma unroll
+    for (int o = LR; o < LR * SPL; o *= 2) {
+      const auto add = [&](T& a) {
+        a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+        a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+      };
+      add(a0), add(a1), add(a2), add(a3);
+    }
+    if (okp && r < nr && lp == 0) {
       T* qp = q + ((int64_t)(out_box ? out_box[b] : b) * npts + p) * C + r;
       qp[0] = a0;
       qp[nr] = a1;
@@ -2004,7 +2013,7 @@ void launch_gather_build(const R* mr, const int32_t* mr_base, const int32_t* mr_
                                                    box_rwg_ptr, box_tri_ptr, sp, gptr_r, gptr_t, gr, gt);
 }
 
-template <typename R, int LR>
+template <typename R, int LR, int SPL>
 static void run_anterp(const R* gr, const R* gt, const int32_t* gptr_r, const int32_t* gptr_t, const int64_t* mr_off,
                        const int64_t* mt_off, const int64_t* box_rwg_ptr, const int64_t* box_tri_ptr, int64_t B,
                        int max_rwg, int max_sc, const int32_t* out_box, const cpx_t<R>* xs, int64_t ldx,
@@ -2015,14 +2024,14 @@ static void run_anterp(const R* gr, const R* gt, const int32_t* gptr_r, const in
   if (ak + at > cap) ak = at = cap / 2;
   const size_t smem = (size_t)(ak + at) * row;
   static SmemAttr attr;
-  smem_attr_once(k_anterp<R, LR>, ANTERP_SMEM, attr.v);
+  smem_attr_once(k_anterp<R, LR, SPL>, ANTERP_SMEM, attr.v);
   // parts of a box's points, up to one pass each, until the blocks fill the
   // chip twice over (4 blocks of 8 warps per SM); a part stages the box again
-  const int64_t npts = (int64_t)sp * sp * sp, passes = ceil_div(npts, 256 / LR);
+  const int64_t npts = (int64_t)sp * sp * sp, passes = ceil_div(npts, 256 / (LR * SPL));
   const int nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(passes, ceil_div(152 * 8, B)));
-  k_anterp<R, LR><<<(unsigned)(B * nsplit), 256, smem, s>>>(gr, gt, gptr_r, gptr_t, mr_off, mt_off, box_rwg_ptr,
-                                                            box_tri_ptr, out_box, xs, ldx, rho, ldr, nr, q, sp, ak, at,
-                                                            nsplit);
+  k_anterp<R, LR, SPL><<<(unsigned)(B * nsplit), 256, smem, s>>>(gr, gt, gptr_r, gptr_t, mr_off, mt_off, box_rwg_ptr,
+                                                                 box_tri_ptr, out_box, xs, ldx, rho, ldr, nr, q, sp,
+                                                                 ak, at, nsplit);
 }
 
 template <typename R>
@@ -2031,13 +2040,20 @@ void launch_anterp(const R* gr, const R* gt, const int32_t* gptr_r, const int32_
                    int max_rwg, int max_sc, const int32_t* out_box, const cpx_t<R>* xs, int64_t ldx,
                    const cpx_t<R>* rho, int64_t ldr, int nr, cpx_t<R>* q, int sp, cudaStream_t s) {
   if (B <= 0 || nr <= 0) return;
-#define EFIE_AN(L)                                                                                                   \
-  run_anterp<R, L>(gr, gt, gptr_r, gptr_t, mr_off, mt_off, box_rwg_ptr, box_tri_ptr, B, max_rwg, max_sc, out_box, xs, \
-                   ldx, rho, ldr, nr, q, sp, s)
-  if (nr == 1) EFIE_AN(1);
-  else if (nr == 2) EFIE_AN(2);
-  else if (nr <= 4) EFIE_AN(4);
-  else EFIE_AN(8);
+#define EFIE_AN(L, S)                                                                                                \
+  run_anterp<R, L, S>(gr, gt, gptr_r, gptr_t, mr_off, mt_off, box_rwg_ptr, box_tri_ptr, B, max_rwg, max_sc, out_box, \
+                      xs, ldx, rho, ldr, nr, q, sp, s)
+  if constexpr (sizeof(R) == 4) {  // FP32 sums keep their order
+    if (nr == 1) EFIE_AN(1, 1);
+    else if (nr == 2) EFIE_AN(2, 1);
+    else if (nr <= 4) EFIE_AN(4, 1);
+    else EFIE_AN(8, 1);
+  } else {
+    if (nr == 1) EFIE_AN(1, 8);
+    else if (nr == 2) EFIE_AN(2, 4);
+    else if (nr <= 4) EFIE_AN(4, 4);
+    else EFIE_AN(8, 2);
+  }
 #undef EFIE_AN
 }
 

@@ -49,3 +49,27 @@ def test_long_axes(case, form):
                     assert err < TOL[form]
     finally:
         h.close()
+
+
+def test_anterpolation_forms():
+    """The FP64 lane forms on boxes whose functions are staged whole (1 to 4 vectors)
+    and in several passes over the sorted lists (8 vectors): 735 RWGs a box."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+    import paper_2606_13482_gb300 as G
+    V, T = E.merge_meshes(E.icosphere(14, 0.4, center=(-1.7, 0.0, 0.0)), E.icosphere(14, 0.4, center=(1.7, 0.3, 0.1)))
+    args = (V, T, 2 * np.pi, 3, 0.2, 1)
+    assert G.plan(*args)[1][0]["n_far_pairs"] > 0
+    X = torch.from_numpy(E.complex_gaussian((8, 3 * len(T) // 2), 5)).cuda()
+    h = G.EFIE(*args, precision=G.EFIE_FP64)
+    try:
+        one = torch.cat([h.matvec(X[r:r + 1].contiguous()) for r in range(8)])
+        for n in (2, 3, 4, 5, 8):
+            y = h.matvec(X[:n].contiguous())
+            # both sum lists of up to some hundred rounded terms in 53 bits
+            assert (y - one[:n]).norm() <= 2.0 ** -53 * 100 * one[:n].norm(), n
+    finally:
+        h.close()
