@@ -1847,9 +1847,11 @@ __global__ void k_gather_build(const R* __restrict__ mr, const int32_t* __restri
 // 0.397 -> 0.078 ms; 48,000 unknowns, FP64, 8 vectors 2.75 -> 1.31 (two passes per 32
 // points before); the nonuniform tree with 22 leaves of 41^3 points on its top
 // level, 64 vectors 166 -> 5.8.  FP64 with lists shared by SPL groups (8 to 16 lanes a
-// point; half or twice as many measured slower on small or on large trees), 1, 2, 4 and
-// 8 vectors: 1,920 unknowns in one level 0.188 -> 0.036, 0.182 -> 0.056, 0.165 -> 0.066,
-// 0.175 -> 0.114; 48,000 unknowns 0.398 -> 0.331, 0.528 -> 0.451, 0.816 -> 0.695, 1.28 -> 1.07.
+// point; half or twice as many measured slower on small or on large trees) and eight
+// entries in flight, 1, 2, 4 and 8 vectors: 1,920 unknowns in one level 0.188 -> 0.032,
+// 0.182 -> 0.051, 0.165 -> 0.053, 0.175 -> 0.094; 48,000 unknowns 0.398 -> 0.300, 0.528 -> 0.400,
+// 0.816 -> 0.638, 1.28 -> 0.98.  FP32, 6,750 unknowns, one vector, eight in flight: 0.081 ->
+// 0.064.
 template <typename R, int LR>
 struct AnterpCfg {
   // values per staged function: rows of 80 bytes (FP32) and 144 (FP64) spread the banks
@@ -1936,13 +1938,27 @@ __global__ void __launch_bounds__(256) k_anterp(const R* __restrict__ gr, const 
         a2.y = fma(m2, xv.y, a2.y);
       };
       if (nchunk == 1) {
-        // every entry belongs to this chunk: four list entries in flight at a time
-        for (; er + 3 * SPL < er1; er += 4 * SPL) {
-          R k_[4], x_[4], y_[4], z_[4];
+        // every entry belongs to this chunk: several list entries in flight.  Eight, the
+        // last ones of a list predicated, in FP64 and with at most two lanes of
+        // vectors; else four (48,000 unknowns, FP32, 8 vectors: 0.195 ms against 0.217)
+        if constexpr (sizeof(R) == 8 || LR <= 2) {
+          for (; er < er1; er += 8 * SPL) {
+            R k_[8], x_[8], y_[8], z_[8];
 #pragma unroll
-          for (int t = 0; t < 4; ++t) load4(er + t * SPL, k_[t], x_[t], y_[t], z_[t]);
+            for (int t = 0; t < 8; ++t)
+              if (er + t * SPL < er1) load4(er + t * SPL, k_[t], x_[t], y_[t], z_[t]);
 #pragma unroll
-          for (int t = 0; t < 4; ++t) mac3((int)k_[t], x_[t], y_[t], z_[t]);
+            for (int t = 0; t < 8; ++t)
+              if (er + t * SPL < er1) mac3((int)k_[t], x_[t], y_[t], z_[t]);
+          }
+        } else {
+          for (; er + 3 * SPL < er1; er += 4 * SPL) {
+            R k_[4], x_[4], y_[4], z_[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) load4(er + t * SPL, k_[t], x_[t], y_[t], z_[t]);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) mac3((int)k_[t], x_[t], y_[t], z_[t]);
+          }
         }
       }
       for (; er < er1; er += SPL) {
