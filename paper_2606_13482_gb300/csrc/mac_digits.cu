@@ -31,11 +31,7 @@ namespace efie {
 
 constexpr int MD_RD = 3;   // groups of 8 sources in the ring
 
-// exponent of one row of n complex values: E with max |value| < 2^E
-__device__ __forceinline__ int md_exponent(int mx) {
-  const int f = mx >> 20;
-  return f == 2047 ? NM_ENAN : f == 0 ? NM_EZERO : f - 1022;
-}
+// exponents of the kernel rows
 __global__ void __launch_bounds__(128) k_spec_rowexp(const double2* __restrict__ K, int64_t O,
                                                      int16_t* __restrict__ kexp) {
   const double2* Kf = K + (int64_t)blockIdx.x * O;
@@ -48,7 +44,7 @@ __global__ void __launch_bounds__(128) k_spec_rowexp(const double2* __restrict__
   for (int d = 16; d > 0; d >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, d));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
-  if (threadIdx.x == 0) kexp[blockIdx.x] = (int16_t)md_exponent(max(max(red[0], red[1]), max(red[2], red[3])));
+  if (threadIdx.x == 0) kexp[blockIdx.x] = (int16_t)nm_row_exponent(max(max(red[0], red[1]), max(red[2], red[3])));
 }
 
 // digits of the source spectra: qd[f][box][c][6] (half2 real, imaginary) and
@@ -66,7 +62,7 @@ __global__ void __launch_bounds__(256) k_spec_digits(const double2* __restrict__
   }
   __syncthreads();
   if (threadIdx.x < C) {
-    const int E = md_exponent(mx[threadIdx.x]);
+    const int E = nm_exponent(mx[threadIdx.x]);
     qexp[f * C + threadIdx.x] = (int16_t)E;
     mx[threadIdx.x] = E;
   }
@@ -232,10 +228,8 @@ k_mac_digits(const double2* __restrict__ K, const int16_t* __restrict__ kexp, co
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         const int c = c0 + 8 * n + 2 * t + (v & 1);
-        const int ex = c < C ? qexp[f * C + c] : NM_EZERO;
-        const int ee = min(max(E + ex - 46, -1022), 1023) + 1023;
-        double sc = __hiloint2double(ee << 20, 0);
-        if (E == NM_ENAN || ex == NM_ENAN) sc = __hiloint2double(0x7ff80000, 0);
+        const NmCol x = nm_col(c < C ? qexp[f * C + c] : 0);
+        const double sc = nm_scale(E, x, 46);
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
           const int q = part * 4 + v;
@@ -248,7 +242,7 @@ k_mac_digits(const double2* __restrict__ K, const int16_t* __restrict__ kexp, co
           const long long T = ((long long)r_[0] << 30) + ((long long)r_[1] << 20) + ((long long)r_[2] << 10) + r_[3];
           const int low = r_[4] + __float2int_rn(fl[n][q] * 0.0009765625f);
           double* ap = acc + (n * 8 + q) * 128;
-          *ap = fma((double)T, sc, fma((double)low, sc * 0.0009765625, *ap));
+          *ap = fma(nm_raise((double)T, x), sc, fma(nm_raise((double)low, x), sc * 0.0009765625, *ap));
           fl[n][q] = 0.f;
         }
       }

@@ -99,8 +99,7 @@ __global__ void k_near_rexp(const void* __restrict__ M, const int64_t* __restric
         const double2 a = Mb[(int64_t)c * nrow];
         mx = max(mx, max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff));
       }
-      const int f = mx >> 20;
-      E = f == 2047 ? NM_ENAN : f == 0 ? NM_EZERO : f - 1022;
+      E = nm_row_exponent(mx);
     } else {
       const float4* Mb = (const float4*)M + blk_off[j] + row;
       int mx = 0;
@@ -139,21 +138,26 @@ __global__ void __launch_bounds__(256) k_near_digits(const double2* __restrict__
       mx = max(mx, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
     }
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  const int f = mx >> 20;
-  const int E = f == 2047 ? NM_ENAN : f == 0 ? NM_EZERO : f - 1022;
+  // a box of subnormal numbers only: its own exponent, the values raised by 2^64
+  const bool sub = (mx >> 20) == 0;
+  const int E = sub ? 32 - __clz(mx) - 1042 : nm_exponent(mx), Ed = sub ? E + 64 : E;
   if (lane == 0) xexp[((int64_t)box * ntt + nt) * 8 + n] = (int16_t)E;
-  const bool zero = r >= nr || f == 0 || f == 2047;
+  const bool zero = r >= nr || E == NM_ENAN;
   const int npair = ((ncol + 7) / 8) * 4;
   for (int cp = lane; cp < npair; cp += 32) {
     const int c = (cp >> 2) * 8 + (cp & 3);
     double2 v0 = make_double2(0, 0), v1 = v0;
     if (!zero && c < ncol) v0 = xr[c];
     if (!zero && c + 4 < ncol) v1 = xr[c + 4];
+    if (sub) {
+      const double up = 18446744073709551616.0;
+      v0 = make_double2(v0.x * up, v0.y * up), v1 = make_double2(v1.x * up, v1.y * up);
+    }
     int a0[NS], a1[NS], b0[NS], b1[NS];
-    nm_digits<NS>(nm_fixed(v0.x, E), a0);
-    nm_digits<NS>(nm_fixed(v0.y, E), b0);
-    nm_digits<NS>(nm_fixed(v1.x, E), a1);
-    nm_digits<NS>(nm_fixed(v1.y, E), b1);
+    nm_digits<NS>(nm_fixed(v0.x, Ed), a0);
+    nm_digits<NS>(nm_fixed(v0.y, Ed), b0);
+    nm_digits<NS>(nm_fixed(v1.x, Ed), a1);
+    nm_digits<NS>(nm_fixed(v1.y, Ed), b1);
     uint2* o = xd + (((kg_off[box] + (cp >> 2)) * ntt + nt) * NS) * 32 + n * 4 + (cp & 3);
 #pragma unroll
     for (int s = 0; s < NS; ++s) o[s * 32] = make_uint2(nm_pack(a0[s], b0[s]), nm_pack(a1[s], b1[s]));
@@ -388,13 +392,11 @@ k_near_mma(const NearMma pa, const NearMma pb, int nr, int ntt, int wk) {
 #pragma unroll
           for (int n = 0; n < NT; ++n) {
             const int xe = __ldg(reinterpret_cast<const int*>(P.xexp + ((int64_t)y * ntt + nt0 + n) * 8) + t);
-            const int xe0 = (int16_t)(xe & 0xffff), xe1 = xe >> 16;
+            const NmCol x0 = nm_col((int16_t)(xe & 0xffff)), x1 = nm_col(xe >> 16);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
-              const int er = v < 2 ? ea : eb, ex = (v & 1) ? xe1 : xe0;
-              const int ee = min(max(er + ex - (F64 ? 46 : 51), -1022), 1023) + 1023;
-              double sc = __hiloint2double(ee << 20, 0);
-              if (er == NM_ENAN || ex == NM_ENAN) sc = __hiloint2double(0x7ff80000, 0);
+              const NmCol xc = (v & 1) ? x1 : x0;
+              const double sc = nm_scale(v < 2 ? ea : eb, xc, F64 ? 46 : 51);
 #pragma unroll
               for (int part = 0; part < 2; ++part) {
                 const int q = part * 4 + v;
@@ -409,10 +411,10 @@ k_near_mma(const NearMma pa, const NearMma pb, int nr, int ntt, int wk) {
                 double* ap = acc + (n * 8 + q) * 128 + tid;
                 if constexpr (F64) {
                   const int low = r_[4] + __float2int_rn(fl[n][q] * 0.0009765625f);
-                  *ap = fma((double)T, sc, fma((double)low, sc * 0.0009765625, *ap));
+                  *ap = fma(nm_raise((double)T, xc), sc, fma(nm_raise((double)low, xc), sc * 0.0009765625, *ap));
                 } else {
                   T = T * 16 + __float2int_rn(fl[n][q] * 0.015625f);
-                  *ap = fma((double)T, sc, *ap);
+                  *ap = fma(nm_raise((double)T, xc), sc, *ap);
                 }
                 fl[n][q] = 0.f;
               }
