@@ -137,11 +137,7 @@ struct FarSet {
   int Rc = 0;
   std::vector<cpx_t<R>*> q, r;
   cpx_t<R>*tmp1 = nullptr, *tmp2 = nullptr, *Qh = nullptr, *Rh = nullptr;
-  // FP64: digits of the source spectra of the largest level for chunks of up to
-  // Rc right-hand sides, and their exponents (optional: without them the
-  // translations run in FP64 arithmetic)
-  uint32_t* qd = nullptr;
-  int16_t* qexp = nullptr;
+  int64_t ntmp = 0;   // values in tmp1 and in tmp2
   // second chunk of a chunk pair (one translation pass per level over 16
   // right-hand sides): its level grids q2[], r2[], and spectra buffers for its
   // sources (Qt2) and results (Rt2)
@@ -631,22 +627,10 @@ void ensure_far_buffers(efie_handle* h, FarSet<R>& F, int Rc) {
   }
   F.tmp1 = h->mem.alloc<cpx_t<R>>(tmax);
   F.tmp2 = h->mem.alloc<cpx_t<R>>(tmax);
+  F.ntmp = tmax;
   F.Qh = h->mem.alloc<cpx_t<R>>(smax);
   F.Rh = h->mem.alloc<cpx_t<R>>(smax);
   F.Rc = Rc;
-  if constexpr (sizeof(R) == 8) {
-    h->mem.release_optional(F.qd);
-    h->mem.release_optional(F.qexp);
-    int64_t nmax = 0, fmax = 0;
-    for (int ell = P.D; ell >= P.top; --ell)
-      if (h->lev[ell - P.top].md.ntiles) {
-        const int64_t n3 = (int64_t)P.L(ell).nfft * P.L(ell).nfft * P.L(ell).nfft;
-        nmax = std::max(nmax, (int64_t)P.L(ell).code.size() * n3);
-        fmax = std::max(fmax, n3);
-      }
-    F.qd = nmax ? h->mem.alloc_optional<uint32_t>(nmax * C * 6) : nullptr;
-    F.qexp = F.qd ? h->mem.alloc_optional<int16_t>(fmax * C) : nullptr;
-  }
 }
 
 void ensure_work(efie_handle* h, int Rw) {
@@ -693,13 +677,9 @@ void drop_digits(efie_handle* h) {
   A.xexp = S.xexp = nullptr;
 }
 
-// the digits of the FP64 spectra, and the translation's tables
+// the tables of the FP64 tensor-core translation
 void drop_mac_digits(efie_handle* h) {
-  if (h->f64.qd) ++h->buf_gen;
-  h->mem.release_optional(h->f64.qd);
-  h->mem.release_optional(h->f64.qexp);
-  h->f64.qd = nullptr;
-  h->f64.qexp = nullptr;
+  ++h->buf_gen;
   for (LevDev& L : h->lev) {
     h->mem.release_optional(const_cast<int32_t*>(L.md.kg_ptr));
     h->mem.release_optional(const_cast<int4*>(L.md.idx));
@@ -1028,9 +1008,10 @@ void run_mac(efie_handle* h, FarSet<R>& F, int ell, int C, const cpx_t<R>* Qin, 
       if constexpr (sizeof(R) == 8)
         // (4 channels of a few thousand tiles: the lists are faster, 0.045 ms against
         // 0.053 for 1,920 unknowns)
-        if (LD.md.ntiles && F.qexp && h->mac_variant != 1 && (C > 4 || LD.md.ntiles * n3 >= 152 * 32)) {
-          launch_mac_digits(Qin, Rout, FL.Kh, LD.md, F.qd, F.qexp, B, C, LD.O, n3, s);
-          ks.launches(1);
+        if (LD.md.ntiles && h->mac_variant != 1 && (C > 4 || LD.md.ntiles * n3 >= 152 * 32)) {
+          // the digits lie in the transforms' intermediates: this level's forward
+          // transform is done with them and its inverse one has not begun
+          ks.launches(launch_mac_digits(Qin, Rout, FL.Kh, LD.md, F.tmp1, F.tmp2, F.ntmp, B, C, LD.O, n3, s) - 1);
           done = true;
         }
       if (!done)

@@ -220,9 +220,10 @@ struct MacDigits {
   const int16_t* kexp = nullptr;    // [nf]
 };
 void launch_spec_rowexp(const double2* K, int64_t nf, int64_t O, int16_t* kexp, cudaStream_t s);
-// qd [nf][B][C][6], qexp [nf][C]: the digits of Q (work space)
-void launch_mac_digits(const double2* Q, double2* Rh, const double2* K, const MacDigits& m, uint32_t* qd, int16_t* qexp,
-                       int64_t B, int C, int64_t O, int64_t nf, cudaStream_t s);
+// tmp1, tmp2: work space of ntmp values each, at least 2 B C (the digits of one
+// frequency) and nf C / 4; returns the number of launches
+int launch_mac_digits(const double2* Q, double2* Rh, const double2* K, const MacDigits& m, double2* tmp1,
+                      double2* tmp2, int64_t ntmp, int64_t B, int C, int64_t O, int64_t nf, cudaStream_t s);
 
 // the six Hessian kernel spectra of the dyadic factorization (ab = 00, 01,
 // 02, 11, 12, 22), [n^3][O] each

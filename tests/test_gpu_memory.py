@@ -1,0 +1,53 @@
+"""Device memory of a handle: what the first FP64 product takes."""
+import numpy as np
+import pytest
+
+import efie_inputs as E
+
+pytestmark = pytest.mark.gpu
+
+K = 2 * np.pi
+
+
+@pytest.fixture(scope="module")
+def G():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as g
+    g.build()
+    import paper_2606_13482_gb300 as G
+    return G
+
+
+def _used():
+    import torch
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free, total = torch.cuda.mem_get_info()
+    return total - free
+
+
+def test_fp64_product_takes_its_grids_and_spectra(G):
+    """Grids, two spectra and two transform intermediates of 8 vectors, and vectors: the digits
+    of the tensor-core translation lie in the intermediates."""
+    import torch
+    args = (*E.icosphere(28, 1.4), K, 3, 0.1, 2)
+    _, lv = G.plan(*args)
+    h = G.EFIE(*args, precision=G.EFIE_FP64)
+    try:
+        x = torch.from_numpy(E.complex_gaussian((8, h.N), 1)).cuda()
+        y = torch.empty_like(x)
+        before = _used()
+        h.matvec(x, y)
+        took = _used() - before
+        C, Nt = 32, 2 * h.N // 3
+        values = sum(2 * L["n_boxes"] * L["sp"] ** 3 * C for L in lv)
+        values += 2 * max(L["n_boxes"] * L["nfft"] ** 3 * C for L in lv)
+        values += 2 * max(max(L["n_boxes"] * L["nfft"] ** 2 * L["sp"] * C for L in lv),
+                          lv[0]["n_boxes"] * lv[1]["sp"] ** 3 * C)   # leaf boxes on the parent's splines
+        values += 8 * (3 * h.N + 3 * Nt)
+        digits = 24 * 8 * 1.3 * (h.N + Nt)       # of the near field's vectors, columns rounded up to 8
+        assert took <= 1.03 * (16 * values + digits), (took, 16 * values, digits)
+    finally:
+        h.close()
