@@ -105,8 +105,7 @@ typedef struct {
                                        pairs; Phi on A's RWG pairs for a direct-factorization
                                        handle) */
     int64_t device_bytes;    /* estimated resident device bytes of the setup products; for a
-                                handle, its device memory without the buffers that only make
-                                products faster and are given back when memory runs short */
+                                handle, all the device memory that it holds now */
     int64_t moment_entries_rwg;  /* leaf moment entries of all RWGs, per vector component */
     int64_t moment_entries_tri;  /* leaf moment entries of the scalar part: triangles (star),
                                     RWG divergences (direct handle) */

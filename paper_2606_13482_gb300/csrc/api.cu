@@ -78,6 +78,14 @@ struct DevMem {
     bytes += b;
     return (T*)p;
   }
+  // room under the limit for b bytes of allocations to come, or an error that
+  // leaves every buffer in place
+  void reserve(int64_t b) {
+    if (limit <= 0 || bytes + b <= limit) return;
+    if (bytes - optional_bytes + b > limit)
+      throw EfieError{EFIE_ENOMEM, "device_mem_limit exceeded (" + std::to_string(bytes - optional_bytes + b) + " bytes)"};
+    drop();
+  }
   // null where the limit or the device has no room
   template <typename T>
   T* alloc_optional(int64_t n) {
@@ -1929,8 +1937,11 @@ int solve_impl(efie_handle* h, const double2* b, double2* x, int n_rhs, double t
   const int max_it = rec ? m * rec_cycles : h->opt.max_iters;
   int cycle = 0;
   Workspace ws{h->mem, {}};
-  double2* Vb = ws.take<double2>((int64_t)n_rhs * (m + 1) * N);
   const bool use_pc = h->net != nullptr && h->opt.precond == EFIE_PRECOND_LEARNED;
+  // basis vectors (and their preconditioned forms), two vectors, coefficients, flags
+  h->mem.reserve(sizeof(double2) * ((int64_t)n_rhs * N * (m + 1 + (use_pc ? m : 0) + 2) +
+                                    (int64_t)2 * n_rhs * (m + 1) + (n_rhs + 1) / 2) + sizeof(int) * (int64_t)n_rhs);
+  double2* Vb = ws.take<double2>((int64_t)n_rhs * (m + 1) * N);
   double2* Zb = use_pc ? ws.take<double2>((int64_t)n_rhs * m * N) : nullptr;
   std::vector<int> pc_fallback(n_rhs, 0);
   double2* wv = ws.take<double2>((int64_t)n_rhs * N);
@@ -2575,7 +2586,7 @@ int efie_num_unknowns(const efie_handle* h, int64_t* n) {
 int efie_plan_info(const efie_handle* h, efie_plan_info_t* info) {
   if (!h || !info) return EFIE_EINVAL;
   fill_plan_info(h->plan, info, nullptr, 0);
-  info->device_bytes = h->mem.bytes - h->mem.optional_bytes;
+  info->device_bytes = h->mem.bytes;
   if (h->direct) {
     // the scalar part is Phi on the RWG pairs of the A blocks, its moments per RWG
     info->near_nnz_V = info->near_nnz_A;

@@ -51,3 +51,46 @@ def test_fp64_product_takes_its_grids_and_spectra(G):
         assert took <= 1.03 * (16 * values + digits), (took, 16 * values, digits)
     finally:
         h.close()
+
+
+def test_device_bytes_counts_the_digits(G):
+    """The digits of a pass of 8 vectors (20 bytes a value and padding) stand in device_bytes in the
+    place of the double-float copies (16 bytes a value) that the other near kernels read."""
+    import torch
+    V, T = E.icosphere(8, 0.5)
+    took = []
+    for variant in (0, 2):
+        h = G.EFIE(V, T, K, 3, 0.1, 2, precision=G.EFIE_MIXED)
+        try:
+            h.autotune_set(8, 0, variant)
+            before = h.info()["device_bytes"]
+            h.matvec(torch.from_numpy(E.complex_gaussian((8, h.N), 2)).cuda())
+            took.append(h.info()["device_bytes"] - before)
+            values = 8 * (h.N + 2 * h.N // 3)
+        finally:
+            h.close()
+    assert 4 * values <= took[0] - took[1] <= 12 * values, (took, values)
+
+
+def test_refused_solve_leaves_the_products_alone(G):
+    """A budget in which a solve's workspace would fit only in part, digits given back or not:
+    refused before anything is given back."""
+    import torch
+    args = (*E.icosphere(8, 0.5), K, 3, 0.1, 2)
+    h = G.EFIE(*args, gmres_restart=1)
+    x = torch.from_numpy(E.complex_gaussian((16, h.N), 3)).cuda()
+    y0 = h.matvec(x)
+    resident = h.info()["device_bytes"]
+    basis = 16 * 2 * h.N * 16          # 16 right-hand sides, 2 basis vectors; as much again for the rest
+    digits = 24 * 8 * (h.N + 2 * h.N // 3)
+    h.close()
+    h = G.EFIE(*args, gmres_restart=1, device_mem_limit=resident + basis * 3 // 2 - digits * 4 // 3)
+    try:
+        assert torch.equal(h.matvec(x), y0)
+        with pytest.raises(G.EfieError) as e:
+            h.solve(x, tol=1e-6)
+        assert e.value.code == -2
+        assert h.info()["device_bytes"] == resident
+        assert torch.equal(h.matvec(x), y0)
+    finally:
+        h.close()
