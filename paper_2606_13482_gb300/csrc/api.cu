@@ -86,6 +86,13 @@ struct DevMem {
       throw EfieError{EFIE_ENOMEM, "device_mem_limit exceeded (" + std::to_string(bytes - optional_bytes + b) + " bytes)"};
     drop();
   }
+  // whether b bytes would fit in the place of `old` allocated ones, as far as the
+  // limit and the device's free memory tell (several allocations: 2 MiB of rounding each)
+  bool fits(int64_t b, int64_t old) const {
+    if (limit > 0 && bytes - old + b > limit) return false;
+    size_t free = 0, total = 0;
+    return cudaMemGetInfo(&free, &total) == cudaSuccess && (int64_t)free + old >= b + (8 << 20);
+  }
   // null where the limit or the device has no room
   template <typename T>
   T* alloc_optional(int64_t n) {
@@ -713,16 +720,23 @@ void drop_near_mma(efie_handle* h) {
 }
 
 // Whether the tensor-core near field takes nr right-hand sides on `s`, with its
-// digit buffers in place.  They are optional: where the memory limit leaves no
-// room for them, and while `s` is being captured, the products go without.
+// digit buffers in place.  They are optional: where the memory limit or the device
+// has no room for them, and while `s` is being captured, the products go without.
+// Smaller ones are given back only where the new ones fit in their place: products
+// that run passes of several sizes would otherwise free and allocate in every pass.
 bool ensure_digits(efie_handle* h, int nr, cudaStream_t s) {
   if (!h->near_mma || nr > near_mma_max_nr(!h->near_df) || (h->near_df && h->near_variant != 0)) return false;
   const int ntt = near_mma_ntiles8(nr);
   if (h->dig_ntt >= ntt) return true;
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;
-  drop_digits(h);
   const int64_t per = 32 * (int64_t)ntt * near_mma_digits(!h->near_df), NL = h->plan.n_leaves;
+  const auto bytes = [&](int64_t n) {  // of buffers for n groups of 8 right-hand sides
+    const int64_t one = NL * 8 * n * (int64_t)sizeof(int16_t);
+    return (h->nkgA + (h->direct ? 0 : h->nkgS)) * (per / ntt * n) * (int64_t)sizeof(uint2) + (h->direct ? one : 2 * one);
+  };
+  if (!h->mem.fits(bytes(ntt), bytes(h->dig_ntt))) return false;
+  drop_digits(h);
   NearMma &A = h->nmA, &S = h->nmS;
   A.xd = h->mem.alloc_optional<uint2>(h->nkgA * per);
   A.xexp = A.xd ? h->mem.alloc_optional<int16_t>(NL * 8 * ntt) : nullptr;

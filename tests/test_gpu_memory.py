@@ -94,3 +94,37 @@ def test_refused_solve_leaves_the_products_alone(G):
         assert torch.equal(h.matvec(x), y0)
     finally:
         h.close()
+
+
+def test_digits_that_do_not_fit_are_not_tried_again(G):
+    """A budget with room for the digits of 8 vectors but not of 64: products of 72, a pass of 64
+    and one of 8, keep the smaller digits instead of giving them back and making them again
+    (which waits for the device)."""
+    import time
+
+    import torch
+    args = (*E.icosphere(28, 1.4), K, 3, 0.1, 2)   # two levels that take pairs of 8-vector chunks
+    h = G.EFIE(*args, precision=G.EFIE_MIXED)
+    h.autotune_set(8, 0, 2)              # double-float copies of the vectors, no digits
+    x = torch.from_numpy(E.complex_gaussian((72, h.N), 5)).cuda()
+    y = torch.empty_like(x)
+    y0 = h.matvec(x)
+    # digits of 64 and of 8 vectors take 20 bytes a value, beside the copies' 16 of 64 vectors, and
+    # 5 to 20% for columns rounded up to 8
+    values = h.N + 2 * h.N // 3
+    limit = h.info()["device_bytes"] + 266 * values
+    h.close()
+    h = G.EFIE(*args, precision=G.EFIE_MIXED, device_mem_limit=limit)
+    try:
+        for _ in range(2):
+            h.matvec(x, y)
+        torch.cuda.synchronize()
+        assert limit - h.info()["device_bytes"] < 106 * values     # the digits of 8 are there
+        t0 = time.perf_counter()
+        torch.cuda._sleep(10 ** 9)       # about half a second
+        h.matvec(x, y)
+        t = time.perf_counter() - t0
+        assert t < 0.2, t
+        assert float((y - y0).norm() / y0.norm()) < 1e-11
+    finally:
+        h.close()
