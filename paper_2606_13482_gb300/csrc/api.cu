@@ -365,6 +365,9 @@ struct efie_handle {
   int max_tset = 0;       // triangles of the largest leaf's triangle set
   // counts the (re)allocations of buffers that captured products refer to
   int64_t buf_gen = 0;
+  // products have been recorded by a caller's stream capture: a replay reads their
+  // optional buffers, which therefore stay until the handle is closed
+  bool captured = false;
 };
 
 namespace {
@@ -682,12 +685,14 @@ void drop_digits(efie_handle* h) {
   if (h->dig_ntt) ++h->buf_gen;
   h->dig_ntt = 0;
   NearMma &A = h->nmA, &S = h->nmS;
-  if (S.xd != A.xd) {
-    h->mem.release_optional(const_cast<uint2*>(S.xd));
-    h->mem.release_optional(const_cast<int16_t*>(S.xexp));
+  if (!h->captured) {
+    if (S.xd != A.xd) {
+      h->mem.release_optional(const_cast<uint2*>(S.xd));
+      h->mem.release_optional(const_cast<int16_t*>(S.xexp));
+    }
+    h->mem.release_optional(const_cast<uint2*>(A.xd));
+    h->mem.release_optional(const_cast<int16_t*>(A.xexp));
   }
-  h->mem.release_optional(const_cast<uint2*>(A.xd));
-  h->mem.release_optional(const_cast<int16_t*>(A.xexp));
   A.xd = S.xd = nullptr;
   A.xexp = S.xexp = nullptr;
 }
@@ -735,7 +740,7 @@ bool ensure_digits(efie_handle* h, int nr, cudaStream_t s) {
     const int64_t one = NL * 8 * n * (int64_t)sizeof(int16_t);
     return (h->nkgA + (h->direct ? 0 : h->nkgS)) * (per / ntt * n) * (int64_t)sizeof(uint2) + (h->direct ? one : 2 * one);
   };
-  if (!h->mem.fits(bytes(ntt), bytes(h->dig_ntt))) return false;
+  if (!h->mem.fits(bytes(ntt), h->captured ? 0 : bytes(h->dig_ntt))) return false;
   drop_digits(h);
   NearMma &A = h->nmA, &S = h->nmS;
   A.xd = h->mem.alloc_optional<uint2>(h->nkgA * per);
@@ -1316,6 +1321,11 @@ void do_matvec(efie_handle* h, const double2* x, int64_t ldx, double2* y, double
     *reinterpret_cast<volatile int*>(h->err_host) = 0;
     throw EfieError{EFIE_ETIMEOUT, "a bounded device wait of an earlier product expired"};
   }
+  if (!h->captured) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();  // (the launches will report it)
+    h->captured = st != cudaStreamCaptureStatusNone;
+  }
   // right-hand sides per far pass: at most 8; the FP64 pass of a mixed handle
   // (true residuals) runs one at a time to bound its buffers
   int Rc = h->opt.rhs_chunk > 0 ? std::min(h->opt.rhs_chunk, 8) : 8;
@@ -1849,7 +1859,9 @@ void setup_impl(efie_handle* h, const efie_mesh* mesh, double k, int p, double g
     }
     // tables of the tensor-core near field; without room for them the products
     // run on the other near kernels
-    M.drop = [h] { drop_near_mma(h); };
+    M.drop = [h] {
+      if (!h->captured) drop_near_mma(h);
+    };
     bool room = true;
     const auto up = [&](const auto& v) {
       using T = typename std::decay<decltype(v[0])>::type;
@@ -3191,9 +3203,11 @@ int efie_batch_matvec(efie_batch* b, const void* const* x, void* const* y, const
       for (size_t i = 0; i < n; ++i) {
         efie_handle* h = b->hs[i];
         cuda_check(cudaStreamWaitEvent(b->streams[i], b->fork, 0), "fork wait");
+        const bool captured = h->captured;
         if (kn[i] > 0)
           do_matvec(h, (const double2*)x[i], h->plan.g.N, (double2*)y[i], nullptr, nullptr, h->plan.g.N, kn[i],
                     false, b->streams[i]);
+        h->captured = captured;  // this graph is captured again when a member's buffers have gone (key_gen)
         cuda_check(cudaEventRecord(b->events[i], b->streams[i]), "join");
         cuda_check(cudaStreamWaitEvent(c, b->events[i], 0), "join wait");
       }

@@ -128,3 +128,43 @@ def test_digits_that_do_not_fit_are_not_tried_again(G):
         assert float((y - y0).norm() / y0.norm()) < 1e-11
     finally:
         h.close()
+
+
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
+def test_captured_product_keeps_its_buffers(G, form):
+    """A caller's CUDA graph of a product, and then a solve that would fit if the digits were given
+    back: it is refused, and the replay still computes the product."""
+    import torch
+    args = (*E.icosphere(8, 0.5), K, 3, 0.1, 2)
+    kw = dict(precision=G.EFIE_FP64 if form == "fp64" else G.EFIE_MIXED, gmres_restart=30)
+    x = None
+    resident = 0
+    for limit in (0, 1):
+        # room for the basis and two vectors if some 260 kB of the 510 kB and more of digits went
+        work = 33 * 16 * 1920 - (1 << 18)
+        h = G.EFIE(*args, device_mem_limit=limit and resident + work, **kw)
+        try:
+            x = torch.from_numpy(E.complex_gaussian((8, h.N), 6)).cuda()
+            y = torch.empty_like(x)
+            y0 = h.matvec(x)
+            resident = h.info()["device_bytes"]
+            if not limit:
+                continue
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                h.matvec(x, y)
+            b = h.rhs_planewave([0, 0, -1.0], [1.0, 0, 0])
+            with pytest.raises(G.EfieError) as e:
+                h.solve(b, tol=1e-6)
+            assert e.value.code == -2 and h.info()["device_bytes"] == resident
+            y.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(y, y0)
+            x.mul_(2.0)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(y, 2.0 * y0)
+        finally:
+            torch.cuda.synchronize()
+            h.close()
