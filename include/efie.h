@@ -272,7 +272,9 @@ int efie_plan_info(const efie_handle *h, efie_plan_info_t *info);
 int efie_rwg_edges(const efie_handle *h, int32_t *edge_vertices, int32_t *tri_pm);
 
 /* Plane-wave right-hand sides [e^i]_m = int f_m . pol_r exp(-jk khat_r . x) dS
- * (Sec. II), FP64.  khat, pol: host [n_rhs][3]; rhs: device c128 [n_rhs][N]. */
+ * (Sec. II), FP64.  khat, pol: host [n_rhs][3]; rhs: device c128 [n_rhs][N].
+ * Calls with more than 64 waves sum in another order, so that a wave's last
+ * bits can differ from those of a shorter call. */
 int efie_rhs_planewave(efie_handle *h, int n_rhs, const double *khat, const double *pol,
                        void *rhs, void *stream);
 

@@ -2998,12 +2998,14 @@ void launch_rhs_planewave(const RhsGeom& g, const double* khat, const double* po
                           cudaStream_t s) {
   int64_t total = g.N * nr;
   if (total <= 0) return;
-  // More waves than one chunk of a product has vectors: by leaf box where its
+  // More waves than one pass of a product has vectors: by leaf box where its
   // triangles' integrals fit in shared memory, up to 8 waves at a time (46 KB: no
   // opt-in, four blocks per SM).  65 waves, 58,080 unknowns: 22.9 ms direct, 2.4 by
-  // box.  Fewer waves keep every bit of the direct sums: they are what products and
-  // solves take as vectors, an FP32 product rounds them, and a last bit of a component
-  // on a rounding boundary moves that product by up to 3e-9.
+  // box.  The line is no crossover of times: fewer waves keep every bit of the direct
+  // sums that callers have had, because an FP32 product rounds them as vectors, and a
+  // last bit of a component on a rounding boundary moves that product by up to 3e-9.
+  // Longer sweeps differ from the direct sums in their last bits, with the same error
+  // against exact values (5.4e-15 against 5.3e-15).
   const int64_t per = 2 * sizeof(double2) * (int64_t)g.max_tset;
   const int W = (int)std::min<int64_t>(std::min(nr, 8), 46 * 1024 / std::max<int64_t>(per, 1));
   if (nr > RHS_DIRECT && W >= 1 && g.n_boxes > 0 && (nr + W - 1) / W <= 65535) {

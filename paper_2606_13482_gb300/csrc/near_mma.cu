@@ -7,15 +7,16 @@
 // 10-bit digits (an error-free fixed-point splitting, Ozaki et al. 2012) and
 // digit products run as FP16 MMAs with FP32 accumulation, which are exact:
 //
-//   a = 2^(EA + 1) sum_i a_i 2^(-9 - 10 i),  |a_0| <= 256, |a_i| <= 512,
+//   a = 2^(EA + 1) sum_i a_i 2^(-9 - 10 i),  |a_0| <= 256, |a_i| <= 512
 //
-// with one exponent EA per (block, row) of the matrix (found at setup) and one
+// (double-float entries: a = 2^EA sum_i a_i 2^(-9 - 10 i), |a_i| <= 512, the first digit too;
+// x has the form above in both), with one exponent EA per (block, row) of the matrix (found at setup) and one
 // exponent EX per (source box, right-hand side) of x.  NS = 5 digits (50 bits
 // below the row's largest entry) stand for the double-float entries of mixed
 // handles, NS = 6 (60 bits) for FP64 ones.  The sum over a group of 8 complex
-// columns of one digit pair is at most 16 * 512 * 512 = 2^22, so an MMA (or a
-// chain of two pairs that hold a top digit, 2^21 each) started from the
-// accumulator 1.5 * 2^23 returns its exact integer sum in the low bits of the
+// columns of one digit pair is at most 16 * 512 * 512 = 2^22, so an MMA (or, with FP64
+// entries, a chain of the two pairs that hold a top digit, 2^21 each; with double-float ones
+// that chain would reach 1.5 * 2^22) started from the accumulator 1.5 * 2^23 returns its exact integer sum in the low bits of the
 // FP32 result, and one integer add moves it to a 32-bit running sum.  Pairs of
 // equal weight i + j share a running sum: weights 0..3 exactly, weight 4 (and 5)
 // in an FP32 accumulator whose rounding lies 2^-58 below the row maximum.  At
