@@ -18,7 +18,8 @@
 // fragments into a ring of its own by asynchronous copies: no barriers.
 //
 // Measured, 4-wavelength sphere, 8 vectors, ms: top level 31.1 -> 4.2 (27.8 from the
-// lists in FP64 arithmetic), leaf level 7.7 -> 3.1; one vector 4.2 -> 1.2 and 1.2 -> 0.84.
+// lists in FP64 arithmetic), leaf level 7.7 -> 3.1 (6.7 for both with the digits in
+// slabs, below); one vector 4.2 -> 1.2 and 1.2 -> 0.84.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -41,8 +41,8 @@
 // waiting on one another half of the time.
 //
 // Measured there, A and the scalar part together, ms (before: double-float on
-// the FP32 pipes, or FP64 arithmetic): 64 vectors 4.0 (33), 16 1.1 (7.3), 8 0.78
-// (4.6); FP64 handles, 8 vectors, 1.2 (13.3).
+// the FP32 pipes, or FP64 arithmetic): 64 vectors 4.1 (33), 16 1.1 (7.3), 8 0.80
+// (4.6); FP64 handles, 8 vectors, 1.4 (13.3).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
