@@ -168,3 +168,55 @@ def test_captured_product_keeps_its_buffers(G, form):
         finally:
             torch.cuda.synchronize()
             h.close()
+
+
+@pytest.mark.parametrize("form,tol", [("fp64", 1e-13), ("mixed", 1e-11)])
+def test_products_without_digits(G, form, tol):
+    """A budget just short of the digits: the products run on the other near kernels and agree."""
+    import torch
+    args = (*E.icosphere(8, 0.5), K, 3, 0.1, 1)
+    kw = dict(precision=G.EFIE_FP64 if form == "fp64" else G.EFIE_MIXED)
+    h = G.EFIE(*args, **kw)
+    x = torch.from_numpy(E.complex_gaussian((8, h.N), 7)).cuda()
+    y0 = h.matvec(x)
+    values, resident = h.N + 2 * h.N // 3, h.info()["device_bytes"]
+    h.close()
+    h = G.EFIE(*args, device_mem_limit=resident - 8 * values, **kw)
+    try:
+        y1 = h.matvec(x)
+        # 24 (FP64) or 20 bytes a value and vector less, the 16 of the double-float copies more
+        less = 8 * values * (24 if form == "fp64" else 20 - 16)
+        assert h.info()["device_bytes"] <= resident - less
+        assert not torch.equal(y1, y0) and float((y1 - y0).norm() / y0.norm()) < tol
+    finally:
+        h.close()
+
+
+def test_batch_after_a_member_grew(G):
+    """A captured batch, then a product of one member that makes its buffers anew: the next batch
+    call is recorded again on the new buffers."""
+    import torch
+    hs = [G.EFIE(*E.icosphere(28, 1.4), K, 3, 0.1, 2, precision=G.EFIE_MIXED),
+          G.EFIE(*E.icosphere(6, 0.4), K, 3, 0.1, 1, precision=G.EFIE_MIXED)]
+    b = G.Batch(hs)
+    try:
+        xs = [torch.from_numpy(E.complex_gaussian((1, h.N), 8 + i)).cuda() for i, h in enumerate(hs)]
+        ys = [torch.empty_like(x) for x in xs]
+        ref = [h.matvec(x) for h, x in zip(hs, xs)]
+        for _ in range(2):
+            b.matvec(xs, ys)
+            torch.cuda.synchronize()
+            assert all(torch.equal(y, r) for y, r in zip(ys, ref))
+        before = hs[0].info()["device_bytes"]
+        hs[0].matvec(torch.from_numpy(E.complex_gaussian((64, hs[0].N), 10)).cuda())
+        assert hs[0].info()["device_bytes"] > before
+        for y in ys:
+            y.zero_()
+        b.matvec(xs, ys)
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, r) for y, r in zip(ys, ref))
+    finally:
+        torch.cuda.synchronize()
+        b.close()
+        for h in hs:
+            h.close()
